@@ -36,7 +36,8 @@ size_t fullpass_smem_bytes(int np, int k, int n);
 cudaError_t launch_fullpass(int np, const float* X, long long m, int n, const float* C, int k,
                             const double* sel_f, int W, int* labels, Globals* g, float gB, float gp2,
                             int incumbent, int grid, cudaStream_t st);
-cudaError_t launch_prepass(const float* v, long long count, Globals* g, int grid, cudaStream_t st);
+cudaError_t launch_prepass(const float* v, long long count, Globals* g, const float* C, int k, int n, int np,
+                           float* Cp, int sms, cudaStream_t st);
 cudaError_t launch_pad(const float* src, long long rows, int n, int np, float* dst, cudaStream_t st);
 cudaError_t launch_unpad(const float* src, long long rows, int n, int np, float* dst, cudaStream_t st);
 cudaError_t launch_select_unpad(const float* Cw, const double* sel_f, int W, int k, int n, int np,
@@ -964,7 +965,7 @@ bm_status bm_fit_create(const float* X_dev, int64_t m, int32_t n, int32_t k, con
     if ((s = alloc_workspace(c, pol.workers))) { delete c; return s; }
     cudaError_t e;
     if ((e = launch_init_state(c->fhat, pol.workers, c->deg, (long long)pol.workers * k, c->glob, c->st)) ||
-        (e = launch_prepass(X_dev, m * n, c->glob, 2 * sm_count(), c->st)) ||
+        (e = launch_prepass(X_dev, m * n, c->glob, nullptr, 0, 0, 0, nullptr, sm_count(), c->st)) ||
         (e = launch_globaltimer(c->timer, c->st))) {
         bm_fit_destroy(c);
         return fail(BM_ECUDA, "launch failed: %s", cudaGetErrorString(e));
@@ -1561,9 +1562,7 @@ bm_status bm_gather(const float* X_dev, int64_t m, int32_t n, const int64_t* idx
 static bm_status stage_sample_and_centroids(bm_fit_ctx* c, const float* S_dev, long long s, const float* C_dev,
                                             int k) {
     CU(launch_pad(S_dev, s, c->n, c->np, c->S, c->st));
-    CU(launch_pad(C_dev, k, c->n, c->np, c->Cw, c->st));
-    CU(launch_prepass(S_dev, s * c->n, c->glob, 2 * sm_count(), c->st));
-    CU(launch_prepass(C_dev, (long long)k * c->n, c->glob, 1, c->st));
+    CU(launch_prepass(S_dev, s * c->n, c->glob, C_dev, k, c->n, c->np, c->Cw, sm_count(), c->st));
     return BM_OK;
 }
 
@@ -1644,9 +1643,7 @@ bm_status bm_assign(const float* X_dev, int64_t m, int32_t n, const float* C_dev
     }
     cudaError_t e;
     if ((e = cudaMemsetAsync(g, 0, sizeof(Globals), sm)) ||
-        (e = launch_pad(C_dev, k, n, np, Cp, sm)) ||
-        (e = launch_prepass(X_dev, m * n, g, 2 * sm_count(), sm)) ||
-        (e = launch_prepass(C_dev, (long long)k * n, g, 1, sm)) ||
+        (e = launch_prepass(X_dev, m * n, g, C_dev, k, n, np, Cp, sm_count(), sm)) ||
         (ev[0] && (e = cudaEventRecord(ev[0], sm))) ||
         (e = launch_fullpass(np, X_dev, m, n, Cp, k, nullptr, 1, labels_out_dev, g, gB, gp2, 0, sm_count(), sm)) ||
         (ev[1] && (e = cudaEventRecord(ev[1], sm)))) {
@@ -1719,7 +1716,7 @@ static bm_status assign_bf16(const void* Xb_dev, const float* norms_dev, const f
     cert_constants(64, gB, gp2);                   // rows of the precision form are 64 wide
     cudaError_t e;
     if ((e = cudaMemsetAsync(g, 0, sizeof(Globals), sm)) ||
-        (e = launch_prepass(C_dev, (long long)k * n, g, 1, sm)) ||
+        (e = launch_prepass(C_dev, (long long)k * n, g, nullptr, 0, 0, 0, nullptr, sm_count(), sm)) ||
         (e = launch_tc_fullpass(Xb_dev, norms_dev, X_dev, m, n, C_dev, k, tau, certify, labels_out_dev, queue, g,
                                 gp2, sm_count(), sm))) {
         cudaFreeAsync(base, sm);

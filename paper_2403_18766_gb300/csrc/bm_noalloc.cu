@@ -24,8 +24,8 @@ size_t fullpass_smem_bytes(int np, int k, int n);
 cudaError_t launch_fullpass(int np, const float* X, long long m, int n, const float* C, int k,
                             const double* sel_f, int W, int* labels, Globals* g, float gB, float gp2,
                             int incumbent, int grid, cudaStream_t st);
-cudaError_t launch_prepass(const float* v, long long count, Globals* g, int grid, cudaStream_t st);
-cudaError_t launch_pad(const float* src, long long rows, int n, int np, float* dst, cudaStream_t st);
+cudaError_t launch_prepass(const float* v, long long count, Globals* g, const float* C, int k, int n, int np,
+                           float* Cp, int sms, cudaStream_t st);
 bm_status status_from_flags(const Globals& h);
 }  // namespace bm
 
@@ -104,9 +104,7 @@ extern "C" bm_status bm_assign_noalloc(const float* X_dev, int64_t m, int32_t n,
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     // The scratch keeps the previous call's contents: clear the accumulators.
     if ((e = cudaMemsetAsync(g, 0, sizeof(bm::Globals), st)) ||
-        (e = bm::launch_pad(C_dev, k, n, np, Cp, st)) ||
-        (e = bm::launch_prepass(X_dev, (long long)m * n, g, 2 * sms, st)) ||
-        (e = bm::launch_prepass(C_dev, (long long)k * n, g, 1, st)) ||
+        (e = bm::launch_prepass(X_dev, (long long)m * n, g, C_dev, k, n, np, Cp, sms, st)) ||
         (e = bm::launch_fullpass(np, X_dev, m, n, Cp, k, nullptr, 1, labels_out_dev, g, gB, gp2, 0, sms, st)))
         return err(BM_ECUDA, "full pass launch: %s", cudaGetErrorString(e));
     bm::Globals h;

@@ -37,38 +37,103 @@ constexpr int kTcK = 64;               // packed row width (BF16 elements)
 
 // ------------------------------------------------------------------ pack
 // Xb[r][chunk c ^ (r & 7)] holds elements 8c .. 8c+7 of row r (BF16, RN);
-// rows m .. m_pad-1 and elements n .. 63 are zero.  norms[r] = fl(sum x_b^2).
+// rows m .. m_pad-1 and elements n .. 63 are zero.  norms[r] = fl(sum x_b^2)
+// as an FMA chain over ascending d; norms[m_pad] = max |x|.
 // Xb may be NULL: the norms (and the max |x|) alone.
-__global__ void pack_bf16_kernel(const float* __restrict__ X, long long m, int n, long long m_pad,
-                                 __nv_bfloat16* __restrict__ Xb, float* __restrict__ norms) {
-    const long long total = Xb ? m_pad * (kTcK / 8) : 0;       // 16-byte chunks (none: norms only)
-    for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < total;
-         e += (long long)gridDim.x * blockDim.x) {
-        const long long r = e / (kTcK / 8);
-        const int c = (int)(e % (kTcK / 8));
-        __align__(16) __nv_bfloat16 v[8];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            const int d = 8 * c + i;
-            v[i] = __float2bfloat16_rn((r < m && d < n) ? X[r * n + d] : 0.f);
-        }
-        const int pc = c ^ (int)(r & 7);
-        *reinterpret_cast<uint4*>(Xb + r * kTcK + 8 * pc) = *reinterpret_cast<const uint4*>(v);
-    }
+//
+// Bound by HBM: 4 n B read, 128 + 4 B written per row.  A CTA of 128 threads
+// takes tiles of 128 rows, which are contiguous in X: the tile is read with
+// coalesced 16-byte loads (all of a thread's loads in flight) into shared
+// memory rows an odd number of 16-byte units apart, each thread packs one row
+// from there (so the norm's chain stays in a thread, and reads and writes of
+// shared memory meet no bank conflicts: the swizzle spreads the chunks), and
+// the packed tile, 16 KB in one piece of Xb, is written with coalesced 16-byte
+// stores.  6 CTAs per SM overlap one another's phases.
+// Measured on 10^7 x 64 (3.88 GB moved): 2,677 us when every thread read its
+// own pieces of rows and the norms came from a second walk, now 589 us (6.6
+// TB/s).
+constexpr int kPkRows = 128;
+constexpr int kPkStride = kTcK + 4;
+__global__ void __launch_bounds__(kPkRows) pack_bf16_kernel(const float* __restrict__ X, long long m, int n,
+                                                            long long m_pad, __nv_bfloat16* __restrict__ Xb,
+                                                            float* __restrict__ norms) {
+    __shared__ __align__(16) float xs[kPkRows * kPkStride];
+    const int tid = threadIdx.x;
+    const bool vec = (n & 3) == 0 && (reinterpret_cast<uintptr_t>(X) & 15) == 0;
+    const int per = vec ? n >> 2 : n;                     // load units per row
+    // e / per for e < 2^13 by multiplication: (2^20 / per rounded up) e 2^-20
+    const unsigned inv = ((1u << 20) + per - 1) / per;
     unsigned int mx = 0;
-    for (long long r = (long long)blockIdx.x * blockDim.x + threadIdx.x; r < m_pad;
-         r += (long long)gridDim.x * blockDim.x) {
-        float acc = 0.f;
-        for (int d = 0; d < n && r < m; ++d) {
-            const float x = X[r * n + d];
-            mx = max(mx, __float_as_uint(x) & 0x7fffffffu);
-            const float b = __bfloat162float(__float2bfloat16_rn(x));
-            acc = __fmaf_rn(b, b, acc);
+    for (int i = tid; i < kPkRows * kPkStride; i += kPkRows) xs[i] = 0.f;      // columns n .. 63
+    for (long long tile = blockIdx.x; tile < m_pad / kPkRows; tile += gridDim.x) {
+        const long long r0 = tile * kPkRows;
+        const int rows = (int)min((long long)kPkRows, m - r0);
+        const float* src = X + r0 * n;
+        __syncthreads();                                  // the previous tile's packed rows are out
+        if (vec) {
+            constexpr int U = kTcK / 4;                   // units per thread at n = 64
+            float4 w[U];
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int e = tid + u * kPkRows;
+                if (u < per) w[u] = e < rows * per ? __ldg(reinterpret_cast<const float4*>(src) + e)
+                                                   : make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+#pragma unroll
+            for (int u = 0; u < U; ++u) {
+                const int e = tid + u * kPkRows;
+                if (u < per) {
+                    const int r = (int)((unsigned)e * inv >> 20);
+                    *reinterpret_cast<float4*>(xs + r * kPkStride + 4 * (e - r * per)) = w[u];
+                }
+            }
+        } else {
+            for (int e = tid; e < kPkRows * per; e += kPkRows) {
+                const int r = (int)((unsigned)e * inv >> 20);
+                xs[r * kPkStride + e - r * per] = e < rows * per ? __ldg(src + e) : 0.f;
+            }
         }
-        norms[r] = acc;
+        __syncthreads();
+        // row tid: norm, max, packed chunks (kept in registers until every
+        // row of the tile has been read)
+        uint4 pk[kTcK / 8];
+        float acc = 0.f;
+#pragma unroll
+        for (int c = 0; c < kTcK / 8; ++c) {
+            const float4 a = *reinterpret_cast<const float4*>(xs + tid * kPkStride + 8 * c);
+            const float4 b = *reinterpret_cast<const float4*>(xs + tid * kPkStride + 8 * c + 4);
+            const float x[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+            __align__(16) __nv_bfloat16 v[8];
+#pragma unroll
+            for (int i = 0; i < 8; ++i) {
+                mx = max(mx, __float_as_uint(x[i]) & 0x7fffffffu);
+                v[i] = __float2bfloat16_rn(x[i]);
+                const float f = __bfloat162float(v[i]);
+                acc = __fmaf_rn(f, f, acc);
+            }
+            pk[c] = *reinterpret_cast<const uint4*>(v);
+        }
+        norms[r0 + tid] = acc;
+        if (Xb) {
+            __syncthreads();
+            uint4* ps = reinterpret_cast<uint4*>(xs);
+#pragma unroll
+            for (int c = 0; c < kTcK / 8; ++c) ps[tid * 8 + (c ^ (tid & 7))] = pk[c];
+            __syncthreads();
+            uint4* dst = reinterpret_cast<uint4*>(Xb + r0 * kTcK);
+#pragma unroll
+            for (int u = 0; u < kTcK / 8; ++u) dst[tid + u * kPkRows] = ps[tid + u * kPkRows];
+            if (n < kTcK) {                               // the staged chunks covered the zero columns
+                __syncthreads();
+                for (int i = tid; i < kPkRows * kTcK / 4; i += kPkRows)
+                    reinterpret_cast<float4*>(xs)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
+            }
+        }
     }
     // norms[m_pad] = max |x| (bits; non-finite values compare above all finite ones)
-    if (mx) atomicMax(reinterpret_cast<unsigned int*>(norms + m_pad), mx);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) mx = max(mx, __shfl_down_sync(0xffffffffu, mx, o));
+    if ((tid & 31) == 0 && mx) atomicMax(reinterpret_cast<unsigned int*>(norms + m_pad), mx);
 }
 
 // ------------------------------------------------------- shape and layout
@@ -546,11 +611,15 @@ size_t tc_smem_bytes(int k) {
 
 cudaError_t launch_pack_bf16(const float* X, long long m, int n, long long m_pad, void* Xb, float* norms,
                              cudaStream_t st) {
-    const long long total = std::max<long long>(m_pad * (kTcK / 8) * (Xb ? 1 : 0), m_pad);
-    const int grid = (int)std::min<long long>(8192, (total + 255) / 256);
     cudaError_t e = cudaMemsetAsync(norms + m_pad, 0, sizeof(float), st);
     if (e != cudaSuccess) return e;
-    pack_bf16_kernel<<<grid, 256, 0, st>>>(X, m, n, m_pad, (__nv_bfloat16*)Xb, norms);
+    int per_sm = 0, dev = 0, sms = 0;
+    if ((e = cudaGetDevice(&dev)) != cudaSuccess ||
+        (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess ||
+        (e = blocks_per_sm((const void*)pack_bf16_kernel, kPkRows, 0, &per_sm)) != cudaSuccess)
+        return e;
+    const long long grid = std::min<long long>(m_pad / kPkRows, (long long)sms * std::max(per_sm, 1));
+    pack_bf16_kernel<<<(unsigned)grid, kPkRows, 0, st>>>(X, m, n, m_pad, (__nv_bfloat16*)Xb, norms);
     return cudaGetLastError();
 }
 
