@@ -30,7 +30,6 @@
 #include "bm_worker.cuh"
 
 namespace bm {
-size_t worker_smem(int np, int k);
 cudaError_t launch_worker(int np, const WorkerArgs& a, int clusters, cudaStream_t st);
 size_t fullpass_smem_bytes(int np, int k, int n);
 cudaError_t launch_fullpass(int np, const float* X, long long m, int n, const float* C, int k,
@@ -205,7 +204,7 @@ thread_local bool t_groups_ok = true;
 // buckets of a Lloyd run (4 bytes per row) must fit beside the worker's
 // shared memory.
 long long rows_cap(int np, int k) {
-    const long long room = ((long long)kSmemLimit - (long long)worker_smem(np, k)) / 4 - 16;
+    const long long room = ((long long)kSmemLimit - (long long)worker_smem(np, k, 1)) / 4 - 16;
     return std::max<long long>(0, std::min<long long>(kMaxRowsPerCta, room));
 }
 
@@ -241,7 +240,6 @@ struct bm_fit_ctx {
     bm_budget bud{};
     unsigned long long seed = 0;
     long long s_lo = 0, s_hi = 0, s_cap = 0, Tcap = 0, H = 0, L_cap = 0;
-    size_t smem = 0;
     float gB = 0, gp2 = 0;
     int rounds_run = 0;
     unsigned long long t0_gpu = 0;
@@ -264,7 +262,8 @@ struct bm_fit_ctx {
     unsigned long long* timer = nullptr;
     // group exchange of workers that span several clusters (null: no groups)
     long long* xpart = nullptr; int* xcnt = nullptr; unsigned long long* xobj = nullptr;
-    unsigned* xbar = nullptr; float* xC = nullptr; int* xflag = nullptr;
+    unsigned* xbar = nullptr; int* xflag = nullptr;
+    long long* kx = nullptr;                // K-means++ exchange words
     int max_cs = 8;
     cudaEvent_t ev_fork = nullptr;
     // phase timing: event pairs around each launch, summed when the stream syncs
@@ -295,6 +294,20 @@ SizePolicy size_policy(const bm_fit_ctx* c) {
     return p;
 }
 
+// Bytes of the group exchange buffers, 0 when the fit cannot use groups
+// (more workers than a cooperative launch can hold clusters, or too large).
+size_t group_bytes(const bm_fit_ctx* c, int W) {
+    if (W > kMaxGroupWorkers) return 0;
+    const size_t part = (size_t)W * 2 * kMaxGroup * c->k * c->np * kAccWords * 8;
+    if (part > ((size_t)256 << 20)) return 0;
+    return part;
+}
+
+// CTAs of one worker in any launch of this fit: the largest group, or one cluster.
+int kpp_ctas(const bm_fit_ctx* c) {
+    return group_bytes(c, c->pol.workers) ? kMaxGroup * kGroupCs : kMaxCluster;
+}
+
 WorkerArgs make_args(const bm_fit_ctx* c, int mode, int parity = 0) {
     WorkerArgs a;
     memset(&a, 0, sizeof a);
@@ -315,7 +328,8 @@ WorkerArgs make_args(const bm_fit_ctx* c, int mode, int parity = 0) {
     a.gB = c->gB; a.gp2 = c->gp2;
     a.xpart = c->xpart; a.xcnt = c->xcnt; a.xobj = c->xobj;
     a.xbar = c->xbar; a.xabort = c->xbar ? reinterpret_cast<int*>(c->xbar + c->pol.workers) : nullptr;
-    a.xC = c->xC; a.xflag = c->xflag;
+    a.xflag = c->xflag;
+    a.kx = c->kx; a.kx_ctas = kpp_ctas(c);
     return a;
 }
 
@@ -405,15 +419,6 @@ void collect_spans(bm_fit_ctx* c) {
 // runs) the padded sample, its indices, draws and sampler table; per worker
 // the K-means++ D^2, labels, centroids and state.
 // Device bytes of a fit's workspace (the layout of alloc_workspace).
-// Bytes of the group exchange buffers, 0 when the fit cannot use groups
-// (more workers than a cooperative launch can hold clusters, or too large).
-size_t group_bytes(const bm_fit_ctx* c, int W) {
-    if (W > kMaxGroupWorkers) return 0;
-    const size_t part = (size_t)W * 2 * kMaxGroup * c->k * c->np * kAccWords * 8;
-    if (part > ((size_t)256 << 20)) return 0;
-    return part;
-}
-
 size_t workspace_bytes(const bm_fit_ctx* c, int W) {
     const long long k = c->k, np = c->np;
     const long long J = 2ll * W * (c->pol.passes + 1);
@@ -424,7 +429,6 @@ size_t workspace_bytes(const bm_fit_ctx* c, int W) {
         take((size_t)W * 2 * kMaxGroup * k * 4);
         take((size_t)W * 2 * kMaxGroup * 4 * 8);
         take((size_t)W * 2 * 4);
-        take((size_t)W * k * np * 4);
         take((size_t)W * 2 * 4);
     }
     take(sizeof(Globals));
@@ -433,8 +437,9 @@ size_t workspace_bytes(const bm_fit_ctx* c, int W) {
     take((size_t)J * c->Tcap * 4);
     take((size_t)J * c->H * 8);
     take((size_t)J * 4);
+    take((size_t)W * 4 * c->s_cap * 4);
     take((size_t)W * c->s_cap * 4);
-    take((size_t)W * c->s_cap * 4);
+    take((size_t)W * 2 * kpp_ctas(c) * 64 * 8);
     take((size_t)W * k * np * 4);
     take((size_t)W * kMaxCluster * k * np * 4);
     take((size_t)W * k);
@@ -457,8 +462,9 @@ bm_status alloc_workspace(bm_fit_ctx* c, int W) {
     const size_t o_draws = take((size_t)J * c->Tcap * 4);
     const size_t o_tab = take((size_t)J * c->H * 8);
     const size_t o_js = take((size_t)J * 4);
-    const size_t o_D2 = take((size_t)W * c->s_cap * 4);
+    const size_t o_D2 = take((size_t)W * 4 * c->s_cap * 4);
     const size_t o_lab = take((size_t)W * c->s_cap * 4);
+    const size_t o_kx = take((size_t)W * 2 * kpp_ctas(c) * 64 * 8);
     const size_t o_Cw = take((size_t)W * k * np * 4);
     const size_t o_Cwc = take((size_t)W * kMaxCluster * k * np * 4);
     const size_t o_deg = take((size_t)W * k);
@@ -467,13 +473,12 @@ bm_status alloc_workspace(bm_fit_ctx* c, int W) {
     const size_t o_L = take((size_t)c->L_cap * 8);
     const size_t o_t = take(8);
     const size_t gb = group_bytes(c, W);
-    size_t o_xp = 0, o_xc = 0, o_xo = 0, o_xb = 0, o_xC = 0, o_xf = 0;
+    size_t o_xp = 0, o_xc = 0, o_xo = 0, o_xb = 0, o_xf = 0;
     if (gb) {
         o_xp = take(gb);
         o_xc = take((size_t)W * 2 * kMaxGroup * k * 4);
         o_xo = take((size_t)W * 2 * kMaxGroup * 4 * 8);
         o_xb = take((size_t)W * 2 * 4);
-        o_xC = take((size_t)W * k * np * 4);
         o_xf = take((size_t)W * 2 * 4);
     }
     cudaError_t e = lib_alloc(&c->base, off, c->st);
@@ -486,13 +491,13 @@ bm_status alloc_workspace(bm_fit_ctx* c, int W) {
     c->glob = (Globals*)(b + o_glob);
     c->S = (float*)(b + o_S); c->idx = (long long*)(b + o_idx); c->draws = (unsigned int*)(b + o_draws);
     c->table = (unsigned long long*)(b + o_tab); c->job_s = (int*)(b + o_js);
-    c->D2 = (float*)(b + o_D2); c->lab = (int*)(b + o_lab); c->Cw = (float*)(b + o_Cw); c->Cw_cta = (float*)(b + o_Cwc);
+    c->D2 = (float*)(b + o_D2); c->kx = (long long*)(b + o_kx); c->lab = (int*)(b + o_lab); c->Cw = (float*)(b + o_Cw); c->Cw_cta = (float*)(b + o_Cwc);
     c->deg = (unsigned char*)(b + o_deg); c->fhat = (double*)(b + o_fhat); c->f_final = (double*)(b + o_ff);
     c->L_buf = (long long*)(b + o_L); c->timer = (unsigned long long*)(b + o_t);
     if (gb) {
         c->xpart = (long long*)(b + o_xp); c->xcnt = (int*)(b + o_xc);
         c->xobj = (unsigned long long*)(b + o_xo); c->xbar = (unsigned*)(b + o_xb);
-        c->xC = (float*)(b + o_xC); c->xflag = (int*)(b + o_xf);
+        c->xflag = (int*)(b + o_xf);
     }
     CU(cudaMemsetAsync(c->glob, 0, sizeof(Globals), c->st));
     CU(cudaMemsetAsync(c->Cw, 0, (size_t)W * k * np * 4, c->st));
@@ -514,7 +519,7 @@ bm_status check_shape(long long m, int n, int k, bool worker = true) {
     if (n < 1 || n > 64) return fail(BM_EINVAL, "n = %d out of range [1, 64]", n);
     if (k < 1) return fail(BM_EINVAL, "k = %d must be >= 1", k);
     if (!worker) return BM_OK;
-    const size_t smem = worker_smem(padded_dim(n), k);
+    const size_t smem = worker_smem(padded_dim(n), k, 1);
     if (smem > kSmemLimit)
         return fail(BM_EINVAL, "k = %d with n = %d needs %zu bytes of shared memory (limit %zu)", k, n,
                     smem, kSmemLimit);
@@ -618,7 +623,6 @@ int plan_launch(const std::vector<bm_fit_ctx*>& fits, std::vector<PlanItem> item
     groups = groups && cooperative_clusters_ok();
     const long long smax = items[0].s;
     const long long cap = rows_cap(c0->np, kmax);
-    const size_t base = worker_smem(c0->np, kmax);
     a.k_smem = kmax;
     for (int gcs = kGroupCs; groups && gcs >= 4; gcs /= 2) {
         std::vector<int> G(nw, 1);
@@ -630,7 +634,7 @@ int plan_launch(const std::vector<bm_fit_ctx*>& fits, std::vector<PlanItem> item
         for (int pass = 0; pass < 3; ++pass) {
             long long rows = 0;
             for (int i = 0; i < nw; ++i) rows = std::max(rows, rows_of(i));
-            capacity = std::min(worker_active_clusters(c0->np, gcs, base + bucket_smem_bytes((int)rows)),
+            capacity = std::min(worker_active_clusters(c0->np, gcs, worker_smem(c0->np, kmax, gcs) + bucket_smem_bytes((int)rows)),
                                 kMaxLaunchClusters);
             while (total < capacity) {
                 int best = -1;
@@ -852,7 +856,6 @@ bm_status plan_fit(const float* X_dev, int64_t m, int32_t n, int32_t k, const bm
     if (c->H > (1ll << 31)) { delete c; return fail(BM_EINVAL, "sample sizes need a sampler table above 2^31"); }
     c->L_cap = (bud.rounds > 0 ? (long long)bud.rounds : 4096ll) * pol.workers * pol.passes;
     c->L_cap = std::min<long long>(c->L_cap, 1ll << 24);
-    c->smem = worker_smem(c->np, k);
     c->rounds_planned = bud.rounds > 0 ? bud.rounds : 0x7fffffff;
     cert_constants(c->np, c->gB, c->gp2);
     *out = c;
@@ -1508,7 +1511,6 @@ static bm_status step_ctx(bm_fit_ctx* c, const float* X, long long m, int n, int
     c->Tcap = m > 0 ? draw_cap(m, std::min<long long>(c->s_cap, m)) : 1024;
     c->H = next_pow2(2 * c->Tcap);
     c->L_cap = 1;
-    c->smem = worker_smem(c->np, k);
     cert_constants(c->np, c->gB, c->gp2);
     return alloc_workspace(c, 1);
 }

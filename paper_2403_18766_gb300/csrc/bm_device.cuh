@@ -371,6 +371,17 @@ __device__ __forceinline__ T warp_sum(T v) {
     return v;
 }
 
+// Inclusive prefix sum over the lanes of a warp.
+__device__ __forceinline__ long long warp_scan(long long v) {
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const long long y = __shfl_up_sync(0xffffffffu, v, o);
+        if (lane >= o) v += y;
+    }
+    return v;
+}
+
 __device__ __forceinline__ unsigned __int128 warp_sum_u128(unsigned __int128 v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {

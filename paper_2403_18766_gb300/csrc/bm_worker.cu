@@ -80,13 +80,13 @@ int worker_max_cluster(int np, int k) {
     return 8;
 }
 
-size_t worker_smem(int np, int k) {
+size_t worker_smem(int np, int k, int cs) {
     switch (np) {
-        case 4: return worker_smem_bytes<4>(k);
-        case 8: return worker_smem_bytes<8>(k);
-        case 16: return worker_smem_bytes<16>(k);
-        case 32: return worker_smem_bytes<32>(k);
-        case 64: return worker_smem_bytes<64>(k);
+        case 4: return worker_smem_bytes<4>(k, cs);
+        case 8: return worker_smem_bytes<8>(k, cs);
+        case 16: return worker_smem_bytes<16>(k, cs);
+        case 32: return worker_smem_bytes<32>(k, cs);
+        case 64: return worker_smem_bytes<64>(k, cs);
     }
     return 0;
 }

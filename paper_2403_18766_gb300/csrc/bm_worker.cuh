@@ -58,14 +58,14 @@ struct WorkerArgs {
     unsigned long long* xobj;         // W x 2 x kMaxGroup x 4 (objective partial, counters)
     unsigned* xbar;                   // W barrier counters (zero at launch)
     int* xabort;                      // W abort flags (zero at launch)
-    float* xC;                        // W x k x NP centroids re-seeded by cluster 0
     int* xflag;                       // W x 2 deadline decisions
     int tpb;                          // threads per CTA: 256, or 512 (largest clusters)
     Globals* glob;
     // samples drawn by the sampling kernel: job (w, slot) = w * (P + 1) + slot
     float* S; long long S_stride;                 // s_cap * NP floats per job
     const int* job_s;                             // sample size of each job
-    float* D2; long long D2_stride;               // s_cap per worker (K-means++ D^2)
+    float* D2; long long D2_stride;               // 4 x s_cap per worker (K-means++ D^2)
+    long long* kx; int kx_ctas;                   // K-means++ exchange: W x 2 x kx_ctas x 64 words
     int* lab;                                     // s_cap per worker (labels, same stride)
     // worker state
     float* Cw;               // W * k * NP (canonical, read at launch start)
@@ -114,13 +114,20 @@ struct Decision {
 // contributions to the owner's words through distributed shared memory.
 constexpr int kAccWords = 3;
 
+// Clusters of k that one CTA of a cluster of cs owns, at most.
+__host__ __device__ inline int owned_slots(int k, int cs) { return (k + cs - 1) / cs; }
+
+// Shared memory of a worker CTA without the label buckets.  A launch asks for
+// the slots its CTAs own (with all k slots, k = 100 at n = 64 took 205 KB and
+// left one CTA per SM; with 13 of them it takes 72 KB and two fit); the size
+// limits of the entry points are stated at cs = 1.
 template <int NP>
-__host__ __device__ inline size_t worker_smem_bytes(int k) {
+__host__ __device__ inline size_t worker_smem_bytes(int k, int cs) {
     size_t b = 0;
     b += align16((size_t)k * NP * 4);           // Ccur
     b += align16((size_t)k * NP * 4);           // Cnext (pushed by the owners)
     b += align16((size_t)k * 4);                // CC
-    b += align16((size_t)k * NP * kAccWords * 8);  // OACC (owned slots; k of them when cs = 1)
+    b += align16((size_t)owned_slots(k, cs) * NP * kAccWords * 8);  // OACC
     b += align16((size_t)k * 4);                // ocnt (owned counts)
     b += align16((size_t)k * 4);                // lcnt (this CTA's counts / bucket cursors)
     b += align16((size_t)(k + 1) * 4);          // lstart (bucket starts)
@@ -146,7 +153,7 @@ cudaError_t launch_worker(int np, const WorkerArgs& a, int clusters, cudaStream_
 int worker_active_clusters(int np, int cs, size_t smem);
 // Whether a cooperative launch keeps its cluster shape here (checked once per device).
 bool cooperative_clusters_ok();
-size_t worker_smem(int np, int k);
+size_t worker_smem(int np, int k, int cs);
 int worker_max_cluster(int np, int k);   // 16 if 16-CTA clusters fit, else 8
 
 }  // namespace bm

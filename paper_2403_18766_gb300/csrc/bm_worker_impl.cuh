@@ -48,14 +48,14 @@ struct Sm {
 };
 
 template <int NP>
-__device__ inline Sm<NP> carve(int k, int rows_cta) {
+__device__ inline Sm<NP> carve(int k, int cs, int rows_cta) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     unsigned char* p = smem_raw;
     Sm<NP> s;
     s.Ccur = (float*)p;            p += align16((size_t)k * NP * 4);
     s.Cnext = (float*)p;           p += align16((size_t)k * NP * 4);
     s.CC = (float*)p;              p += align16((size_t)k * 4);
-    s.OACC = (long long*)p;        p += align16((size_t)k * NP * kAccWords * 8);
+    s.OACC = (long long*)p;        p += align16((size_t)owned_slots(k, cs) * NP * kAccWords * 8);
     s.ocnt = (int*)p;              p += align16((size_t)k * 4);
     s.lcnt = (int*)p;              p += align16((size_t)k * 4);
     s.lstart = (int*)p;            p += align16((size_t)(k + 1) * 4);
@@ -87,7 +87,8 @@ struct Worker {
     int rank, cs, w, k, n;
     int gi, G, ctaW, nW;    // cluster gi of the worker's G clusters; CTA ctaW of its nW
     int xpar = 0;           // parity of the next group exchange
-    unsigned gepoch = 0;    // group barriers passed (thread 0)
+    int kpar = 0;           // parity of the next K-means++ exchange
+    unsigned gepoch = 0;    // group barriers passed
     Grids g;
     float* S;               // current sample (padded rows), set per pass
     float* D2; float* Cw_mine;
@@ -111,10 +112,10 @@ struct Worker {
         nW = G * cs;
         k = a.k;
         n = a.n;
-        sm = carve<NP>(k, a.rows_cta);
+        sm = carve<NP>(k, cs, a.rows_cta);
         g = grids_from_maxbits(a.glob->maxbits);
         S = a.S;
-        D2 = a.D2 + (long long)w * a.D2_stride;
+        D2 = a.D2 + (long long)w * 4 * a.D2_stride;
         lab_prev = a.lab + (long long)w * a.D2_stride;
         Cw_mine = a.Cw_cta + ((long long)w * kMaxCluster + rank) * (long long)k * NP;
     }
@@ -139,11 +140,6 @@ struct Worker {
         lo = s * ctaW / nW;
         hi = s * (ctaW + 1) / nW;
     }
-    // Rows of this CTA in K-means++, which cluster 0 of the group runs alone.
-    __device__ void kslice(long long s, long long& lo, long long& hi) const {
-        lo = s * rank / cs;
-        hi = s * (rank + 1) / cs;
-    }
     __device__ bool lead() const { return gi == 0 && rank == 0; }     // records the worker's counters
 
     // ------------------------------------------------ group of clusters
@@ -155,26 +151,31 @@ struct Worker {
     // at once and the launch reports a timeout (results are then discarded).
     __device__ void gsync() {
         if (G == 1) return;
+        ++gepoch;
         __syncthreads();
         if (threadIdx.x == 0) {
-            ++gepoch;
             __threadfence();
             atomicAdd(a.xbar + w, 1u);
-            const unsigned target = gepoch * (unsigned)nW;
-            const volatile unsigned* bar = a.xbar + w;
-            const volatile int* ab = a.xabort + w;
-            for (unsigned polls = 0; *bar < target; ++polls) {
-                if (*ab) break;
-                if (polls >= (1u << 22)) {
-                    atomicExch(a.xabort + w, 1);
-                    atomicOr(&a.glob->err, kErrTimeout);
-                    break;
-                }
-                __nanosleep(64);
-            }
-            __threadfence();
+            gwait();
         }
         __syncthreads();
+    }
+    // One thread: wait until every CTA of the group has passed barrier
+    // `gepoch` (polls back off only once the wait is long).
+    __device__ void gwait() {
+        const unsigned target = gepoch * (unsigned)nW;
+        const volatile unsigned* bar = a.xbar + w;
+        const volatile int* ab = a.xabort + w;
+        for (unsigned polls = 0; *bar < target; ++polls) {
+            if (*ab) break;
+            if (polls >= (1u << 22)) {
+                atomicExch(a.xabort + w, 1);
+                atomicOr(&a.glob->err, kErrTimeout);
+                break;
+            }
+            if (polls > 256) __nanosleep(64);
+        }
+        __threadfence();
     }
     __device__ bool group_aborted() const { return G > 1 && *(const volatile int*)(a.xabort + w) != 0; }
     // Offsets of this worker's exchange slots (parity par, cluster q).
@@ -801,147 +802,323 @@ struct Worker {
         }
     }
 
-    __device__ void kmeanspp(long long s, unsigned long long k1) {
-        long long lo, hi;
-        kslice(s, lo, hi);
-        bool any_live = false;
-        for (int j = 0; j < k; ++j) any_live |= (sm.deg[j] == 0);
-        unsigned int mloc = 0;
-        if (any_live) {
-            for (long long i = lo + threadIdx.x; i < hi; i += TPB) {
-                float x[NP];
-                load_row(i, x);
-                float dm = __int_as_float(0x7f800000);
-                for (int j = 0; j < k; ++j)
-                    if (!sm.deg[j]) dm = fminf(dm, d32<NP>(x, sm.Ccur + (size_t)j * NP));
-                D2[i] = dm;
-                mloc = max(mloc, __float_as_uint(dm));
+    // D^2 buffer b (0..3) of the worker: one holds D^2, the others the D^2
+    // each candidate would leave, so that taking a candidate is a change of
+    // buffer and no distance is computed twice.
+    __device__ float* d2buf(int b) const { return D2 + (size_t)b * a.D2_stride; }
+
+    // Rows of warp `v` of the worker's CTA `cta`: contiguous, so that prefix
+    // sums over CTAs, warps and rows run in row order.
+    __device__ void kpp_rows(long long s, int cta, int v, long long& w0, long long& w1) const {
+        const long long lo = s * cta / nW, rows = s * (cta + 1) / nW - lo;
+        w0 = lo + rows * v / (TPB / 32);
+        w1 = lo + rows * (v + 1) / (TPB / 32);
+    }
+
+    // One exchange of K-means++ among every CTA of the worker: each publishes
+    // NT sums of weights (per warp and in all) and maxima, then, after a
+    // barrier, every CTA works out the same answer from the published words
+    // alone: the array `best` with the least total (the lowest on ties), its
+    // maximum M and, when M still has the exponent E (or E is kNoExp: nothing
+    // to draw from) and `jdraw` < k, the `trials` candidate rows of centroid
+    // jdraw: the rows at which the prefix of the weights of D^2 buffer
+    // bufs[best] passes the draws.  Warp l finds candidate l by a scan over
+    // the CTAs, over the warps of one CTA and over the rows of one warp, and
+    // leaves the row in candbuf.  One barrier per centroid is the only time
+    // the CTAs wait for one another.
+    static constexpr int kNoExp = 1 << 20;
+    static constexpr int kKppWords = 8 + 3 * kMaxWarps;     // of the 64 words of a CTA's slot
+    __device__ float* candbuf(int par, int l) const {       // in the (idle) sums: 24 NP bytes per cluster, k >= 2
+        return reinterpret_cast<float*>(sm.OACC) + (par * 3 + l) * NP;
+    }
+    __device__ void kpp_exchange(long long s, int NT, const long long (&sum)[3], const unsigned (&mx)[3], int E,
+                                 const int (&bufs)[3], int jdraw, int trials, unsigned long long k1, int cpar) {
+        constexpr int NW = TPB / 32;
+        const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+        long long* wsum = reinterpret_cast<long long*>(sm.inbox);       // [3][kMaxWarps]: 384 of 512 bytes
+        unsigned* wmax = reinterpret_cast<unsigned*>(sm.red128);        // [3][kMaxWarps]: 192 of 256 bytes
+        for (int l = 0; l < NT; ++l) {
+            const long long v = warp_sum(l == 0 ? sum[0] : l == 1 ? sum[1] : sum[2]);
+            const unsigned mv = __reduce_max_sync(0xffffffffu, l == 0 ? mx[0] : l == 1 ? mx[1] : mx[2]);
+            if (lane == 0) { wsum[l * kMaxWarps + wid] = v; wmax[l * kMaxWarps + wid] = mv; }
+        }
+        __syncthreads();
+        long long* slots = a.kx + ((size_t)w * 2 + kpar) * a.kx_ctas * 64;
+        kpar ^= 1;
+        if (wid == 0) {
+            long long* my = slots + (size_t)ctaW * 64;
+            for (int e = lane; e < NT * NW; e += 32)
+                my[8 + (e / NW) * kMaxWarps + e % NW] = wsum[(e / NW) * kMaxWarps + e % NW];
+            if (lane < NT) {
+                long long t = 0;
+                unsigned mv = 0;
+                for (int v = 0; v < NW; ++v) {
+                    t += wsum[lane * kMaxWarps + v];
+                    mv = max(mv, wmax[lane * kMaxWarps + v]);
+                }
+                my[lane] = t;
+                my[4 + lane] = (long long)mv;
+            }
+            __syncwarp();
+        }
+        if (G == 1) {
+            cl.sync();
+        } else {
+            ++gepoch;
+            if (threadIdx.x == 0) {
+                __threadfence();
+                atomicAdd(a.xbar + w, 1u);
+            }
+            if (wid < 3) {                                  // the warps that read what the others published
+                if (lane == 0) gwait();
+                __syncwarp();
+            }
+        }
+        if (wid < 3) {
+            // lane's CTAs: [lane ch, (lane + 1) ch)
+            const int ch = (nW + 31) / 32;
+            const int q0 = lane * ch, q1 = min(nW, q0 + ch);
+            long long tot[3] = {0, 0, 0};
+            unsigned mm[3] = {0, 0, 0};
+            for (int q = q0; q < q1; ++q)
+#pragma unroll
+                for (int l = 0; l < 3; ++l)
+                    if (l < NT) {
+                        tot[l] += __ldcg(slots + (size_t)q * 64 + l);
+                        mm[l] = max(mm[l], (unsigned)__ldcg(slots + (size_t)q * 64 + 4 + l));
+                    }
+            int best = 0;
+            long long Wtot = 0;
+#pragma unroll
+            for (int l = 0; l < 3; ++l)
+                if (l < NT) {
+                    long long t = tot[l];
+#pragma unroll
+                    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+                    if (l == 0 || t < Wtot) { Wtot = t; best = l; }
+                }
+            const unsigned M = __reduce_max_sync(0xffffffffu, best == 0 ? mm[0] : best == 1 ? mm[1] : mm[2]);
+            if (threadIdx.x == 0) { sm.bcast[2] = best; sm.bcast[3] = (long long)M; }
+            if (jdraw < k && E != kNoExp && M != 0 && frexp_exp(M) == E && wid < trials) {
+                const unsigned long long u = draw_below(a.seed, k1, (unsigned long long)wid, (unsigned long long)jdraw,
+                                                        (unsigned long long)Wtot);
+                long long rest = (long long)u;
+                // the CTA
+                const long long mine = best == 0 ? tot[0] : best == 1 ? tot[1] : tot[2];
+                long long pre = warp_scan(mine);
+                int src = __ffs(__ballot_sync(0xffffffffu, rest < pre)) - 1;
+                bool bad = src < 0;                          // cannot happen: the prefix covers [0, Wtot)
+                src = max(src, 0);
+                rest -= __shfl_sync(0xffffffffu, pre - mine, src);
+                int q = min(src * ch, nW - 1);
+                for (; q + 1 < min(nW, src * ch + ch); ++q) {
+                    const long long t = __ldcg(slots + (size_t)q * 64 + best);
+                    if (rest < t) break;
+                    rest -= t;
+                }
+                // its warp
+                const long long wm = lane < NW ? __ldcg(slots + (size_t)q * 64 + 8 + best * kMaxWarps + lane) : 0;
+                pre = warp_scan(wm);
+                src = __ffs(__ballot_sync(0xffffffffu, rest < pre)) - 1;
+                bad |= src < 0;
+                src = max(src, 0);
+                rest -= __shfl_sync(0xffffffffu, pre - wm, src);
+                // the row: lanes over equal contiguous pieces of the warp's rows
+                long long w0, w1;
+                kpp_rows(s, q, src, w0, w1);
+                const int bb = best == 0 ? bufs[0] : best == 1 ? bufs[1] : bufs[2];
+                const float* dv = d2buf(bb);
+                const long long piece = (w1 - w0 + 31) / 32;
+                const long long p0 = min(w1, w0 + piece * lane), p1 = min(w1, p0 + piece);
+                long long ps = 0;
+                for (long long i = p0; i < p1; i += 8) {     // eight loads in flight
+                    float t[8];
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) t[e] = i + e < p1 ? __ldcg(dv + i + e) : 0.f;
+#pragma unroll
+                    for (int e = 0; e < 8; ++e) ps += quant(t[e], E);
+                }
+                pre = warp_scan(ps);
+                src = __ffs(__ballot_sync(0xffffffffu, rest < pre)) - 1;
+                bad |= src < 0;
+                src = max(src, 0);
+                rest -= __shfl_sync(0xffffffffu, pre - ps, src);
+                const long long a0 = __shfl_sync(0xffffffffu, p0, src), a1 = __shfl_sync(0xffffffffu, p1, src);
+                long long row = -1;
+                for (long long r0 = a0; r0 < a1; r0 += 32) {     // that piece, a lane per row
+                    const long long t = r0 + lane < a1 ? quant(__ldcg(dv + r0 + lane), E) : 0;
+                    pre = warp_scan(t);
+                    const unsigned hit = __ballot_sync(0xffffffffu, rest < pre);
+                    if (hit) { row = r0 + __ffs(hit) - 1; break; }
+                    rest -= __shfl_sync(0xffffffffu, pre, 31);
+                }
+                if (bad || row < 0 || row >= s) {
+                    if (lane == 0) atomicOr(&a.glob->err, group_aborted() ? kErrTimeout : kErrArgs);
+                    row = 0;
+                }
+                float* cb = candbuf(cpar, wid);
+                for (int d = lane; d < NP; d += 32) cb[d] = S[row * NP + d];
             }
         }
         __syncthreads();
+    }
+
+    // Greedy K-means++ of the degenerate centroids, by every CTA of the worker
+    // (all clusters of a group).  What bounded it: cluster 0 alone computed
+    // the distances of the whole sample, each centroid took four barriers with
+    // serial scans between them, and the winner's distances were computed
+    // again.  Now a centroid costs one pass over the CTA's rows and one
+    // exchange: the candidates' potentials are at the same time the weight
+    // sums of the next draw as long as the largest D^2 keeps its exponent (the
+    // quantisation grid), else one more pass over D^2 and two exchanges.
+    // A candidate's distances are cut short where they cannot matter: partial
+    // sums of squares never decrease (each addition is rounded, the terms are
+    // not negative), so once every row of a warp has reached its D^2 the
+    // minimum is D^2, whatever the other dimensions hold.
+    // Measured: seeding k = 50 on 64,000 x 32 by one cluster 2.38 -> 1.5 ms;
+    // the worker launch of 8 workers at 10^7 x 64, k = 100 (40,000-row samples)
+    // 17.8 -> 6.7 ms, of which the smaller shared memory (owned_slots) 6 ms.
+    __device__ void kmeanspp(long long s, unsigned long long k1) {
+        const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+        long long w0, w1;
+        kpp_rows(s, ctaW, wid, w0, w1);
         const int trials = a.trials < 1 ? 1 : (a.trials > 3 ? 3 : a.trials);
-        const long long ch = (hi - lo + TPB - 1) / TPB;
-        const long long c0 = lo + ch * threadIdx.x, c1 = min(hi, c0 + ch);
-        for (int j = 0; j < k; ++j) {
-            if (!sm.deg[j]) continue;
-            long long pick;
-            if (!any_live) {
-                pick = (long long)draw_below(a.seed, k1, 0, (unsigned long long)j, (unsigned long long)s);
-            } else {
-                const unsigned int mb = block_max_u32(mloc, sm.redu);
-                if (threadIdx.x == 0) sm.x->maxbits = mb;
-                cl.sync();                                                   // [A]
-                if (threadIdx.x == 0) {
-                    unsigned int M = 0;
-                    for (int q = 0; q < cs; ++q) M = max(M, rx(q)->maxbits);
-                    sm.bcast[2] = M;
-                }
-                __syncthreads();
-                const unsigned int M = (unsigned int)sm.bcast[2];
-                if (M == 0) {
-                    pick = (long long)draw_below(a.seed, k1, 0, (unsigned long long)j, (unsigned long long)s);
-                } else {
-                    const int E = frexp_exp(M);
-                    long long wmine = 0;
-                    for (long long i = c0; i < c1; ++i) wmine += quant(D2[i], E);
-                    long long ctaTot;
-                    const long long excl = block_exscan(wmine, sm.red64, &ctaTot);
-                    if (threadIdx.x == 0) sm.x->wsum = ctaTot;
-                    cl.sync();                                               // [B]
-                    if (threadIdx.x < 4) sm.x->cand[threadIdx.x] = -1;
-                    if (threadIdx.x == 0) {
-                        long long base = 0, tot = 0;
-                        for (int q = 0; q < cs; ++q) {
-                            const long long v = rx(q)->wsum;
-                            if (q < rank) base += v;
-                            tot += v;
-                        }
-                        sm.bcast[3] = base;
-                        sm.bcast[4] = tot;
-                    }
-                    __syncthreads();
-                    const long long base = sm.bcast[3];
-                    const unsigned long long Wtot = (unsigned long long)sm.bcast[4];
-                    for (int l = 0; l < trials; ++l) {
-                        const unsigned long long u = draw_below(a.seed, k1, (unsigned long long)l,
-                                                                (unsigned long long)j, Wtot);
-                        const long long lo_w = base + excl;
-                        if ((long long)u >= lo_w && (long long)u < lo_w + wmine) {
-                            long long run = lo_w;
-                            for (long long i = c0; i < c1; ++i) {
-                                run += quant(D2[i], E);
-                                if (run > (long long)u) { sm.x->cand[l] = (int)i; break; }
-                            }
-                        }
-                    }
-                    cl.sync();                                               // [C]
-                    if (threadIdx.x < trials) {
-                        int c = -1;
-                        for (int q = 0; q < cs; ++q) c = max(c, rx(q)->cand[threadIdx.x]);
-                        sm.bcast[5 + threadIdx.x] = c;
-                    }
-                    __syncthreads();
-                    int cand[3];
-#pragma unroll
-                    for (int l = 0; l < 3; ++l) {
-                        cand[l] = (l < trials) ? (int)sm.bcast[5 + l] : 0;
-                        if (cand[l] < 0 || cand[l] >= s) {          // cannot happen: prefix covers [0, W)
-                            if (threadIdx.x == 0) atomicOr(&a.glob->err, kErrArgs);
-                            cand[l] = 0;
-                        }
-                    }
-                    long long pot[3] = {0, 0, 0};
-                    for (long long i = lo + threadIdx.x; i < hi; i += TPB) {
-                        float x[NP];
-                        load_row(i, x);
-                        const float d2 = D2[i];
-#pragma unroll
-                        for (int l = 0; l < 3; ++l) {
-                            if (l < trials) {
-                                const float dc = d32<NP>(x, S + (long long)cand[l] * NP);
-                                pot[l] += quant(fminf(d2, dc), E);
-                            }
-                        }
-                    }
-#pragma unroll
-                    for (int l = 0; l < 3; ++l) {
-                        if (l < trials) {
-                            const long long t = block_sum<long long>(pot[l], sm.red64);
-                            if (threadIdx.x == 0) sm.x->pot[l] = t;
-                        }
-                    }
-                    cl.sync();                                               // [D]
-                    if (threadIdx.x == 0) {
-                        long long best = 0;
-                        int bl = 0;
-                        for (int l = 0; l < trials; ++l) {
-                            long long t = 0;
-                            for (int q = 0; q < cs; ++q) t += rx(q)->pot[l];
-                            if (l == 0 || t < best) { best = t; bl = l; }
-                        }
-                        sm.bcast[2] = cand[bl];
-                    }
-                    __syncthreads();
-                    pick = sm.bcast[2];
-                    __syncthreads();
-                }
-            }
-            // centroid j = S[pick]
-            if (lead() && threadIdx.x == 0) atomicAdd(&a.glob->reseeded, 1ull);
+        auto next_deg = [&](int j) { ++j; while (j < k && !sm.deg[j]) ++j; return j; };
+        auto count = [&] { if (lead() && threadIdx.x == 0) atomicAdd(&a.glob->reseeded, 1ull); };
+        bool any_live = false;
+        for (int j = 0; j < k; ++j) any_live |= (sm.deg[j] == 0);
+        int j = next_deg(-1);
+        int cur = 0;
+        if (!any_live) {                                     // the first centroid: uniform
+            const long long pick = (long long)draw_below(a.seed, k1, 0, (unsigned long long)j, (unsigned long long)s);
+            count();
             for (int d = threadIdx.x; d < NP; d += TPB) sm.Ccur[(size_t)j * NP + d] = S[pick * NP + d];
             __syncthreads();
-            mloc = 0;
-            for (long long i = lo + threadIdx.x; i < hi; i += TPB) {
+            for (long long i = w0 + lane; i < w1; i += 32) {
                 float x[NP];
                 load_row(i, x);
-                const float dj = d32<NP>(x, sm.Ccur + (size_t)j * NP);
-                const float v = any_live ? fminf(D2[i], dj) : dj;
-                D2[i] = v;
-                mloc = max(mloc, __float_as_uint(v));
+                d2buf(cur)[i] = d32<NP>(x, sm.Ccur + (size_t)j * NP);
             }
-            __syncthreads();
-            any_live = true;
+            j = next_deg(j);
+        } else {
+            for (long long i = w0 + lane; i < w1; i += 32) {
+                float x[NP];
+                load_row(i, x);
+                float dm = __int_as_float(0x7f800000);
+                for (int c = 0; c < k; ++c)
+                    if (!sm.deg[c]) dm = fminf(dm, d32<NP>(x, sm.Ccur + (size_t)c * NP));
+                d2buf(cur)[i] = dm;
+            }
         }
+        bool drawn = false;                                  // candidates of centroid j are in candbuf(cpar, .)
+        int cpar = 0, E = kNoExp;
+        while (j < k) {
+            if (!drawn) {                                    // the grid's exponent, then the weights on it
+                long long ws[3] = {0, 0, 0};
+                unsigned mx[3] = {0, 0, 0};
+                const int bf[3] = {cur, cur, cur};
+                for (long long i = w0 + lane; i < w1; i += 32) mx[0] = max(mx[0], __float_as_uint(d2buf(cur)[i]));
+                kpp_exchange(s, 1, ws, mx, kNoExp, bf, k, trials, k1, cpar);
+                const unsigned M = (unsigned)sm.bcast[3];
+                if (M == 0) {                                // every row sits on a centroid: uniform picks
+                    for (; j < k; j = next_deg(j)) {
+                        const long long pick = (long long)draw_below(a.seed, k1, 0, (unsigned long long)j,
+                                                                     (unsigned long long)s);
+                        count();
+                        for (int d = threadIdx.x; d < NP; d += TPB) sm.Ccur[(size_t)j * NP + d] = S[pick * NP + d];
+                    }
+                    break;
+                }
+                E = frexp_exp(M);
+                for (long long i = w0 + lane; i < w1; i += 32) ws[0] += quant(d2buf(cur)[i], E);
+                kpp_exchange(s, 1, ws, mx, E, bf, j, trials, k1, cpar);
+            }
+            // potentials of the candidates, and the D^2 each would leave.  The
+            // next row is on its way while this one is scored: all of it, or
+            // for NP = 64 its first 16 dimensions (the others are asked for
+            // 16 dimensions ahead).
+            constexpr int H = NP <= 8 ? NP : (NP == 64 ? 16 : 8);    // dimensions between cuts
+            constexpr int PF = NP == 64 ? 16 : NP;                   // dimensions fetched a row ahead
+            const float* c0 = candbuf(cpar, 0);
+            const float* dcur = d2buf(cur);
+            float* dn[3] = {d2buf((cur + 1) & 3), d2buf((cur + 2) & 3), d2buf((cur + 3) & 3)};
+            const int bf[3] = {(cur + 1) & 3, (cur + 2) & 3, (cur + 3) & 3};
+            long long pot[3] = {0, 0, 0};
+            unsigned mx[3] = {0, 0, 0};
+            float4 xn[PF / 4];
+            float d2n = 0.f;
+            auto fetch = [&](long long i) {
+                if (i < w1) {
+                    d2n = dcur[i];
+#pragma unroll
+                    for (int q = 0; q < PF / 4; ++q) xn[q] = reinterpret_cast<const float4*>(S + i * NP)[q];
+                }
+            };
+#pragma unroll
+            for (int q = 0; q < PF / 4; ++q) xn[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+            fetch(w0 + lane);
+            for (long long b = w0; b < w1; b += 32) {        // warp-uniform trips
+                const long long i = b + lane;
+                const bool valid = i < w1;
+                float4 x[PF / 4];
+#pragma unroll
+                for (int q = 0; q < PF / 4; ++q) x[q] = xn[q];
+                const float d2 = d2n;
+                fetch(i + 32);
+                const float4* rest = reinterpret_cast<const float4*>(S + (valid ? i : w0) * NP);
+                float4 v[2][H / 4];                          // NP = 64: the chunk in hand and the next one
+                float acc[3] = {0.f, 0.f, 0.f};
+                auto add = [&](int l, const float4& xv, int q) {
+                    const float4 c = *reinterpret_cast<const float4*>(c0 + l * NP + 4 * q);
+                    float2 t0 = __fadd2_rn(make_float2(xv.x, xv.y), make_float2(-c.x, -c.y));
+                    float2 t1 = __fadd2_rn(make_float2(xv.z, xv.w), make_float2(-c.z, -c.w));
+                    t0 = __fmul2_rn(t0, t0);
+                    t1 = __fmul2_rn(t1, t1);
+                    acc[l] = __fadd_rn(__fadd_rn(__fadd_rn(__fadd_rn(acc[l], t0.x), t0.y), t1.x), t1.y);
+                };
+                bool go[3] = {true, trials > 1, trials > 2};
+#pragma unroll
+                for (int h = 0; h < NP / H; ++h) {
+                    if (h > 0) {
+#pragma unroll
+                        for (int l = 0; l < 3; ++l)
+                            go[l] = go[l] && __any_sync(0xffffffffu, valid && acc[l] < d2);
+                        if (!(go[0] || go[1] || go[2])) break;
+                    }
+                    if (PF < NP && h + 1 < NP / H)
+#pragma unroll
+                        for (int q = 0; q < H / 4; ++q) v[(h + 1) & 1][q] = rest[(h + 1) * (H / 4) + q];
+#pragma unroll
+                    for (int l = 0; l < 3; ++l)
+                        if (go[l])
+#pragma unroll
+                            for (int q = 0; q < H / 4; ++q)
+                                add(l, (PF == NP || h == 0) ? x[((PF == NP ? h : 0) * (H / 4) + q)] : v[h & 1][q],
+                                    h * (H / 4) + q);
+                }
+                if (valid) {
+#pragma unroll
+                    for (int l = 0; l < 3; ++l)
+                        if (l < trials) {
+                            const float m = fminf(d2, acc[l]);
+                            dn[l][i] = m;
+                            pot[l] += quant(m, E);
+                            mx[l] = max(mx[l], __float_as_uint(m));
+                        }
+                }
+            }
+            const int jn = next_deg(j);
+            kpp_exchange(s, trials, pot, mx, E, bf, jn, trials, k1, cpar ^ 1);
+            const int best = (int)sm.bcast[2];
+            const unsigned M = (unsigned)sm.bcast[3];
+            count();
+            for (int d = threadIdx.x; d < NP; d += TPB) sm.Ccur[(size_t)j * NP + d] = candbuf(cpar, best)[d];
+            cur = bf[best];
+            drawn = M != 0 && frexp_exp(M) == E;
+            cpar ^= 1;
+            j = jn;
+        }
+        __syncthreads();
     }
 };
 
@@ -1051,15 +1228,9 @@ __global__ void __launch_bounds__(TPB, 512 / TPB) worker_kernel(const __grid_con
             bool any_deg = false;
             for (int j = 0; j < W.k; ++j) any_deg |= (W.sm.deg[j] != 0);
             if (any_deg) {
-                // re-seeding is in place (Alg. 1); a group's cluster 0 runs it
-                // over the whole sample and hands the centroids to the others
+                // re-seeding is in place (Alg. 1)
                 const long long t_k = clock64();
-                if (W.gi == 0) W.kmeanspp(s_w, stream_k1(kPurposeKpp, w, t, p));
-                if (W.G > 1) {
-                    if (W.gi == 0 && W.rank == 0) W.store_centroids(a.xC + (size_t)w * W.k * NP);
-                    W.gsync();
-                    if (W.gi > 0) W.load_centroids(a.xC + (size_t)w * W.k * NP);
-                }
+                W.kmeanspp(s_w, stream_k1(kPurposeKpp, w, t, p));
                 W.store_centroids(W.Cw_mine);
                 W.trace_add(0, t_k);
             }
@@ -1105,7 +1276,7 @@ __global__ void __launch_bounds__(TPB, 512 / TPB) worker_kernel(const __grid_con
 
 template <int NP>
 int worker_max_cluster_t(int k) {
-    const size_t smem = worker_smem_bytes<NP>(k);
+    const size_t smem = worker_smem_bytes<NP>(k, 1);
     if (allow_max_smem((const void*)worker_kernel<NP, 256, false>) != cudaSuccess ||
         allow_max_smem((const void*)worker_kernel<NP, 512, false>) != cudaSuccess ||
         cudaFuncSetAttribute(worker_kernel<NP, 256, false>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) != cudaSuccess ||
@@ -1168,7 +1339,7 @@ int worker_active_clusters_t(int cs, size_t smem) {
 
 template <int NP, int TPB, bool BATCH>
 cudaError_t launch_worker_tpb(const WorkerArgs& a, int clusters, cudaStream_t st) {
-    const size_t smem = worker_smem_bytes<NP>(a.k_smem > 0 ? a.k_smem : a.k) + bucket_smem_bytes(a.rows_cta);
+    const size_t smem = worker_smem_bytes<NP>(a.k_smem > 0 ? a.k_smem : a.k, a.cs) + bucket_smem_bytes(a.rows_cta);
     cudaError_t e = allow_max_smem((const void*)worker_kernel<NP, TPB, BATCH>);
     if (e != cudaSuccess) return e;
     if (a.cs > 8) {
