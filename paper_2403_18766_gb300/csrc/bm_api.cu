@@ -38,7 +38,7 @@ cudaError_t launch_fullpass(int np, const float* X, long long m, int n, const fl
 cudaError_t launch_prepass(const float* v, long long count, Globals* g, const float* C, int k, int n, int np,
                            float* Cp, int sms, cudaStream_t st);
 cudaError_t launch_pad(const float* src, long long rows, int n, int np, float* dst, cudaStream_t st);
-cudaError_t launch_unpad(const float* src, long long rows, int n, int np, float* dst, cudaStream_t st);
+cudaError_t launch_unpad(const float* src, long long rows, int n, int np, float* dst, int tiles, cudaStream_t st);
 cudaError_t launch_select_unpad(const float* Cw, const double* sel_f, int W, int k, int n, int np,
                                 float* dst, cudaStream_t st);
 cudaError_t launch_init_state(double* fhat, int W, unsigned char* deg, long long kdeg, Globals* g,
@@ -294,6 +294,9 @@ SizePolicy size_policy(const bm_fit_ctx* c) {
     return p;
 }
 
+// Floats of one sample job: s_cap padded rows, in whole tiles of four.
+long long sample_floats(const bm_fit_ctx* c) { return (c->s_cap + 3) / 4 * 4 * c->np; }
+
 // Bytes of the group exchange buffers, 0 when the fit cannot use groups
 // (more workers than a cooperative launch can hold clusters, or too large).
 size_t group_bytes(const bm_fit_ctx* c, int W) {
@@ -319,7 +322,7 @@ WorkerArgs make_args(const bm_fit_ctx* c, int mode, int parity = 0) {
     a.max_lloyd = c->bud.max_lloyd; a.trials = c->bud.kpp_candidates; a.tol = c->bud.tol;
     a.seed = c->seed;
     a.mode = mode; a.cs = c->cs; a.glob = c->glob;
-    a.S_stride = c->s_cap * c->np;
+    a.S_stride = sample_floats(c);
     a.S = c->S + (long long)parity * c->jobs * a.S_stride;
     a.job_s = c->job_s + (long long)parity * c->jobs;
     a.D2 = c->D2; a.D2_stride = c->s_cap; a.lab = c->lab;
@@ -347,7 +350,7 @@ SampleArgs make_sample_args(bm_fit_ctx* c, int mode, int jobs, int parity = 0) {
     const long long J = (long long)parity * c->jobs +
                         ((mode == kSampleRound) ? (long long)c->w_lo * (c->pol.passes + 1) : 0);
     a.worker_base = (mode == kSampleRound) ? c->w_lo : 0;
-    a.S_stride = c->s_cap * c->np; a.S = c->S + J * a.S_stride;
+    a.S_stride = sample_floats(c); a.S = c->S + J * a.S_stride;
     a.idx_stride = c->s_cap; a.idx = c->idx + J * a.idx_stride;
     a.draws_stride = c->Tcap; a.draws = c->draws + J * a.draws_stride; a.Tcap = c->Tcap;
     a.H = c->H; a.table_stride = c->H; a.table = c->table + J * a.table_stride;
@@ -432,7 +435,7 @@ size_t workspace_bytes(const bm_fit_ctx* c, int W) {
         take((size_t)W * 2 * 4);
     }
     take(sizeof(Globals));
-    take((size_t)J * c->s_cap * np * 4);
+    take((size_t)J * sample_floats(c) * 4);
     take((size_t)J * c->s_cap * 8);
     take((size_t)J * c->Tcap * 4);
     take((size_t)J * c->H * 8);
@@ -457,7 +460,7 @@ bm_status alloc_workspace(bm_fit_ctx* c, int W) {
     size_t off = 0;
     auto take = [&](size_t bytes) { size_t o = off; off += (bytes + 255) & ~(size_t)255; return o; };
     const size_t o_glob = take(sizeof(Globals));
-    const size_t o_S = take((size_t)J * c->s_cap * np * 4);
+    const size_t o_S = take((size_t)J * sample_floats(c) * 4);
     const size_t o_idx = take((size_t)J * c->s_cap * 8);
     const size_t o_draws = take((size_t)J * c->Tcap * 4);
     const size_t o_tab = take((size_t)J * c->H * 8);
@@ -1151,7 +1154,7 @@ bm_status bm_fit_worker_centroids(bm_fit_ctx* c, int32_t w, float* C_out_dev) {
     if (w < c->w_lo || w >= c->w_hi) return fail(BM_EINVAL, "worker %d not in [%d, %d)", w, c->w_lo, c->w_hi);
     bm_status s = check_ptr(C_out_dev, "C_out_dev");
     if (s) return s;
-    CU(launch_unpad(c->Cw + (size_t)w * c->k * c->np, c->k, c->n, c->np, C_out_dev, c->st));
+    CU(launch_unpad(c->Cw + (size_t)w * c->k * c->np, c->k, c->n, c->np, C_out_dev, 0, c->st));
     CU(cudaStreamSynchronize(c->st));
     return BM_OK;
 }
@@ -1555,7 +1558,7 @@ bm_status bm_gather(const float* X_dev, int64_t m, int32_t n, const int64_t* idx
     a.idx_stride = 0;
     a.step_s = s;
     CU(launch_sample(c->np, a, 1, c->st));
-    CU(launch_unpad(c->S, s, n, c->np, S_out_dev, c->st));
+    CU(launch_unpad(c->S, s, n, c->np, S_out_dev, 1, c->st));
     Globals h;
     if ((st = read_globals(c, &h))) return st;
     return status_from_flags(h);
@@ -1583,7 +1586,7 @@ bm_status bm_kmeanspp(const float* S_dev, int64_t s, int32_t n, float* C_inout_d
     WorkerArgs a = make_args(c, kModeStepKpp);
     a.trials = trials; a.step_s = s; a.step_worker = worker; a.step_round = round; a.step_pass = pass;
     CU(launch_worker(c->np, a, 1, c->st));
-    CU(launch_unpad(c->Cw, k, n, c->np, C_inout_dev, c->st));
+    CU(launch_unpad(c->Cw, k, n, c->np, C_inout_dev, 0, c->st));
     Globals h;
     if ((st = read_globals(c, &h))) return st;
     return status_from_flags(h);
@@ -1607,7 +1610,7 @@ bm_status bm_lloyd(const float* S_dev, int64_t s, int32_t n, float* C_inout_dev,
     a.step_f = c->f_final; a.step_iters = (int*)c->L_buf;
     a.step_empty = empty_out_dev ? empty_out_dev : c->deg;
     CU(launch_worker(c->np, a, 1, c->st));
-    CU(launch_unpad(c->Cw, k, n, c->np, C_inout_dev, c->st));
+    CU(launch_unpad(c->Cw, k, n, c->np, C_inout_dev, 0, c->st));
     double f = 0;
     int it = 0;
     CU(cudaMemcpyAsync(&f, c->f_final, 8, cudaMemcpyDeviceToHost, c->st));

@@ -245,7 +245,7 @@ __global__ void __launch_bounds__(kSampleThreads, 1) sample_kernel(const SampleA
         if (threadIdx.x == 0 && a.job_s) a.job_s[job] = (int)s;
         return;
     }
-    // gather (padded rows, zeros in the padding); 16-byte loads when the rows
+    // gather (padded rows in tiles, zeros in the padding); 16-byte loads when the rows
     // of X are 16-byte aligned.  A thread takes kGatherBatch items (16-byte
     // pieces of padded rows) at a time: their row indices, then their loads,
     // are all in flight together, so that a large sample does not pay two
@@ -281,7 +281,7 @@ __global__ void __launch_bounds__(kSampleThreads, 1) sample_kernel(const SampleA
         }
 #pragma unroll
         for (int u = 0; u < U; ++u)
-            if (i0 + u * RS < s) reinterpret_cast<float4*>(S + (i0 + u * RS) * NP)[q] = v[u];
+            if (i0 + u * RS < s) *reinterpret_cast<float4*>(S + tile_at<NP>(i0 + u * RS, 4 * q)) = v[u];
     }
     if (threadIdx.x == 0 && a.job_s) a.job_s[job] = (int)s;
 }

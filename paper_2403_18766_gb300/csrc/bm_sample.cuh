@@ -78,7 +78,7 @@ struct SampleArgs {
     int purpose, worker, rnd, pss;
     long long step_s;
     // per-job buffers
-    float* S; long long S_stride;              // s_cap * NP floats
+    float* S; long long S_stride;              // s_cap rows of NP floats (tile_at)
     long long* idx; long long idx_stride;      // s_cap
     unsigned int* draws; long long draws_stride;
     long long Tcap;

@@ -62,7 +62,7 @@ struct WorkerArgs {
     int tpb;                          // threads per CTA: 256, or 512 (largest clusters)
     Globals* glob;
     // samples drawn by the sampling kernel: job (w, slot) = w * (P + 1) + slot
-    float* S; long long S_stride;                 // s_cap * NP floats per job
+    float* S; long long S_stride;                 // s_cap rows of NP floats per job (tile_at)
     const int* job_s;                             // sample size of each job
     float* D2; long long D2_stride;               // 4 x s_cap per worker (K-means++ D^2)
     long long* kx; int kx_ctas;                   // K-means++ exchange: W x 2 x kx_ctas x 64 words

@@ -135,6 +135,18 @@ struct Worker {
         return a.job_s[job];
     }
 
+    // Elements D0 .. D0 + DN - 1 of sample row i (D0 a multiple of 8 unless NP = 4).
+    template <int D0, int DN>
+    __device__ __forceinline__ void load_chunks(long long i, float4 (&v)[DN / 4]) const {
+        if constexpr (NP == 4) {
+            v[0] = __ldg(reinterpret_cast<const float4*>(S + i * NP));
+        } else {
+            const float* p = S + tile_at<NP>(i, D0);
+#pragma unroll
+            for (int c = 0; c < DN / 8; ++c) ld8(p + c * (NP <= 8 ? 8 : 32), v[2 * c], v[2 * c + 1]);
+        }
+    }
+
     // Rows of this CTA: its share of the worker's G * cs CTAs.
     __device__ void slice(long long s, long long& lo, long long& hi) const {
         lo = s * ctaW / nW;
@@ -310,7 +322,9 @@ struct Worker {
         const int sub = lane / LPR, d0 = lane % LPR;
         const int b0 = (int)((long long)nrows * wid / (TPB / 32));
         const int b1 = (int)((long long)nrows * (wid + 1) / (TPB / 32));
-        const float* Sl = S + lo * NP;
+        int dof[DPL];                                      // offsets of this lane's dimensions in a tile
+#pragma unroll
+        for (int t = 0; t < DPL; ++t) dof[t] = (int)tile_at<NP>(0, d0 + t * LPR);
         bool ok = true;
         int cur = -1;                                      // cluster of this lane's running sum
         long long shi[DPL], slo[DPL];
@@ -332,7 +346,7 @@ struct Worker {
 #pragma unroll
                 for (int t = 0; t < DPL; ++t) {
                     const int d = d0 + t * LPR;
-                    xv[u][t] = (p < b1 && d < n) ? Sl[(long long)r * NP + d] : 0.f;
+                    xv[u][t] = (p < b1 && d < n) ? S[tile_at<NP>(lo + r, 0) + dof[t]] : 0.f;
                 }
             }
         };
@@ -399,6 +413,164 @@ struct Worker {
     // lloyd); mode 2: incremental -- the sums are exact integers, so only rows
     // whose label changed since the previous assignment move from their old
     // cluster to the new one.
+    struct Tally {                       // what the rows of a thread add up to
+        unsigned __int128 f = 0;
+        unsigned int inex = 0, resc = 0;
+        bool ok = true;
+    };
+    // Rows row0 + 32 r + lane (r < R, below hi) of one warp; [nx0, nx1) are
+    // the rows the warp takes next.
+    template <int R>
+    __device__ __forceinline__ void assign_rows(long long row0, long long lo, long long hi, long long nx0, long long nx1,
+                                                int mode, const CertC& cc, Tally& ty) {
+        const float gB = a.gB, gp2 = a.gp2;
+        const int gf = g.gf;
+        const int lane = threadIdx.x & 31;
+        float2 m2x[R][NP / 2];                               // -2 x, dimension pairs
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const long long row = row0 + 32 * r + lane;
+            float4 v[NP / 4];
+#pragma unroll
+            for (int q = 0; q < NP / 4; ++q) v[q] = make_float4(0.f, 0.f, 0.f, 0.f);
+            if (row < hi) load_chunks<0, NP>(row, v);
+#pragma unroll
+            for (int q = 0; q < NP / 4; ++q) {
+                m2x[r][2 * q + 0] = __fmul2_rn(make_float2(-2.f, -2.f), make_float2(v[q].x, v[q].y));
+                m2x[r][2 * q + 1] = __fmul2_rn(make_float2(-2.f, -2.f), make_float2(v[q].z, v[q].w));
+            }
+        }
+        int oldlab[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+            oldlab[r] = (mode == 2 && row0 + 32 * r + lane < hi) ? lab_prev[row0 + 32 * r + lane] : -1;
+        if (nx0 < nx1) {   // start the L2 -> L1 fetch of the warp's next rows (their tiles are contiguous)
+            const char* pn = reinterpret_cast<const char*>(S + tile_at<NP>(nx0, 0));
+            const int bytes = (int)(nx1 - nx0) * NP * 4;
+            for (int o = lane * 128; o < bytes; o += 32 * 128) asm volatile("prefetch.global.L1 [%0];" ::"l"(pn + o));
+            if (mode == 2 && lane * 32 < nx1 - nx0)
+                asm volatile("prefetch.global.L1 [%0];" ::"l"(lab_prev + nx0 + lane * 32));
+        }
+        float g1[R], g2[R];
+        int j1[R];
+#pragma unroll
+        for (int r = 0; r < R; ++r) { g1[r] = __int_as_float(0x7f800000); g2[r] = g1[r]; j1[r] = 0; }
+        for (int j = 0; j < k; ++j) {
+            // g_j = ||c_j||^2 - 2 x.c_j as two interleaved partial sums
+            // (even and odd dimensions, packed FP32 FMA), then added:
+            // NP + 1 terms in another order, inside the certificate's
+            // gamma_{2NP+2} bound.
+            const float* cj = sm.Ccur + (size_t)j * NP;
+            const float ccj = sm.CC[j];
+            float2 e2[R];
+#pragma unroll
+            for (int r = 0; r < R; ++r) e2[r] = make_float2(ccj, 0.f);
+#pragma unroll
+            for (int q = 0; q < NP / 4; ++q) {
+                const float4 cv = reinterpret_cast<const float4*>(cj)[q];
+                const float2 c01 = make_float2(cv.x, cv.y), c23 = make_float2(cv.z, cv.w);
+#pragma unroll
+                for (int r = 0; r < R; ++r) {
+                    e2[r] = __ffma2_rn(m2x[r][2 * q + 0], c01, e2[r]);
+                    e2[r] = __ffma2_rn(m2x[r][2 * q + 1], c23, e2[r]);
+                }
+            }
+            float e[R];
+#pragma unroll
+            for (int r = 0; r < R; ++r) e[r] = __fadd_rn(e2[r].x, e2[r].y);
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                g2[r] = fminf(g2[r], fmaxf(g1[r], e[r]));
+                j1[r] = (e[r] < g1[r]) ? j : j1[r];
+                g1[r] = fminf(g1[r], e[r]);
+            }
+        }
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const long long row = row0 + 32 * r + lane;
+            const bool valid = row < hi;
+            const float xn2 = xnorm2_up_m2x<NP>(m2x[r]);
+            const float xn = __fsqrt_ru(xn2);
+            int lab = 0;
+            float dv = 0.f;
+            if (valid) {
+                if (certified(g1[r], g2[r], xn2, xn, cc, gB, gp2)) {
+                    lab = j1[r];
+                    dv = d32_m2x<NP>(m2x[r], sm.Ccur + (size_t)lab * NP);
+                } else {
+                    ty.resc++;
+                    dv = d32_m2x<NP>(m2x[r], sm.Ccur);
+                    for (int j = 1; j < k; ++j) {
+                        const float dj = d32_m2x<NP>(m2x[r], sm.Ccur + (size_t)j * NP);
+                        if (dj < dv) { dv = dj; lab = j; }
+                    }
+                }
+                acc_obj(ty.f, dv, gf, ty.inex);
+            }
+            if (mode == 1) {
+                if (valid) {
+                    lab_prev[row] = lab;
+                    sm.labs[row - lo] = (unsigned short)lab;
+                    atomicAdd(&sm.lcnt[lab], 1);
+                }
+            } else if (mode == 2) {
+                // Move rows whose label changed between clusters.  Many
+                // movers: each lane moves its own row.  Few movers (later
+                // iterations): the warp moves them one at a time, lanes
+                // over dimensions, so the warp does not walk the move path
+                // with one or two lanes active.
+                const bool moved = valid && oldlab[r] != lab;
+                const unsigned mv = __ballot_sync(0xffffffffu, moved);
+                if (__popc(mv) > 8) {
+                    if (moved) {
+                        // the row is in registers (x = -m2x / 2, exact)
+                        ty.ok &= move_row_lane(m2x[r], oldlab[r], lab, ty.inex);
+                        lab_prev[row] = lab;
+                    }
+                } else {
+                    unsigned rem = mv;
+                    while (rem) {
+                        const int src = __ffs(rem) - 1;
+                        rem &= rem - 1u;
+                        const long long srow = __shfl_sync(0xffffffffu, row, src);
+                        const int snew = __shfl_sync(0xffffffffu, lab, src);
+                        const int sold = __shfl_sync(0xffffffffu, oldlab[r], src);
+                        if (lane == src) {
+                            red_s32(owner_count(snew), 1);
+                            red_s32(owner_count(sold), -1);
+                            lab_prev[srow] = snew;
+                        }
+                                                for (int d = lane; d < n; d += 32) {
+                            __int128 v;
+                            ty.ok &= fixed_of(S[tile_at<NP>(srow, d)], g.gx, ty.inex, v);
+                            add_words(owner_words(snew, d), v);
+                            add_words(owner_words(sold, d), -v);
+                        }
+                    }
+                }
+            }
+        }
+    }
+    // The rows are taken in trips of TPB R rows, R as large as leaves no warp
+    // idle: a short remainder (or a small sample's whole slice) is spread over
+    // all warps instead of filling a few.
+    template <int R>
+    __device__ __forceinline__ bool assign_trip(int want, long long t0, long long t1, int nwant, long long lo,
+                                                long long hi, int mode, const CertC& cc, Tally& ty) {
+        if constexpr (R > 1)
+            if (want < R) return assign_trip<R / 2>(want, t0, t1, nwant, lo, hi, mode, cc, ty);
+        const int wid = threadIdx.x >> 5;
+        const long long row0 = t0 + (long long)wid * 32 * R, nx0 = min(hi, t1 + (long long)wid * 32 * nwant);
+        if (row0 < hi)
+            assign_rows<R>(row0, lo, hi, nx0, min(hi, nx0 + 32 * nwant), mode, cc, ty);
+        return true;
+    }
+    __device__ static int trip_rows(long long left) {        // R for the rows that are left
+        constexpr int RT = RowsPerThread<NP>::v;
+        int R = RT;
+        while (R > 1 && left <= (long long)TPB * (R / 2)) R >>= 1;
+        return R;
+    }
     __device__ void assign_slice(long long s, int mode) {
         constexpr int RT = RowsPerThread<NP>::v;
         long long lo, hi;
@@ -408,148 +580,17 @@ struct Worker {
         __syncthreads();
         const long long t_loop = clock64();
         const CertC cc = *sm.cert;
-        const float gB = a.gB, gp2 = a.gp2;
-        const int gf = g.gf;
-        unsigned __int128 facc = 0;
-        unsigned int inex = 0, resc = 0;
-        bool ok = true;
+        Tally ty;
         const int lane = threadIdx.x & 31;
-        // warp-uniform trip count (the move step below uses warp ballots)
-        for (long long base0 = lo + (long long)(threadIdx.x & ~31) * RT; base0 < hi;
-             base0 += (long long)TPB * RT) {
-            const long long base = base0 + (long long)lane * RT;
-            float2 m2x[RT][NP / 2];                          // -2 x, dimension pairs
-#pragma unroll
-            for (int r = 0; r < RT; ++r) {
-                const long long row = base + r;
-                if (row < hi) {
-                    const float4* p = reinterpret_cast<const float4*>(S + row * NP);
-#pragma unroll
-                    for (int q = 0; q < NP / 4; ++q) {
-                        const float4 v = p[q];
-                        m2x[r][2 * q + 0] = make_float2(-2.f * v.x, -2.f * v.y);
-                        m2x[r][2 * q + 1] = make_float2(-2.f * v.z, -2.f * v.w);
-                    }
-                } else {
-#pragma unroll
-                    for (int d = 0; d < NP / 2; ++d) m2x[r][d] = make_float2(0.f, 0.f);
-                }
-            }
-            int oldlab[RT];
-#pragma unroll
-            for (int r = 0; r < RT; ++r)
-                oldlab[r] = (mode == 2 && base + r < hi) ? lab_prev[base + r] : -1;
-            {   // start the L2 -> L1 fetch of this thread's rows of the next trip
-                const long long nb = base + (long long)TPB * RT;
-                if (nb < hi) {
-                    const char* pn = reinterpret_cast<const char*>(S + nb * NP);
-#pragma unroll
-                    for (int o = 0; o < RT * NP * 4; o += 128)
-                        asm volatile("prefetch.global.L1 [%0];" ::"l"(pn + o));
-                    if (mode == 2) asm volatile("prefetch.global.L1 [%0];" ::"l"(lab_prev + nb));
-                }
-            }
-            float g1[RT], g2[RT];
-            int j1[RT];
-#pragma unroll
-            for (int r = 0; r < RT; ++r) { g1[r] = __int_as_float(0x7f800000); g2[r] = g1[r]; j1[r] = 0; }
-            for (int j = 0; j < k; ++j) {
-                // g_j = ||c_j||^2 - 2 x.c_j as two interleaved partial sums
-                // (even and odd dimensions, packed FP32 FMA), then added:
-                // NP + 1 terms in another order, inside the certificate's
-                // gamma_{2NP+2} bound.
-                const float* cj = sm.Ccur + (size_t)j * NP;
-                const float ccj = sm.CC[j];
-                float2 e2[RT];
-#pragma unroll
-                for (int r = 0; r < RT; ++r) e2[r] = make_float2(ccj, 0.f);
-#pragma unroll
-                for (int q = 0; q < NP / 4; ++q) {
-                    const float4 cv = reinterpret_cast<const float4*>(cj)[q];
-                    const float2 c01 = make_float2(cv.x, cv.y), c23 = make_float2(cv.z, cv.w);
-#pragma unroll
-                    for (int r = 0; r < RT; ++r) {
-                        e2[r] = __ffma2_rn(m2x[r][2 * q + 0], c01, e2[r]);
-                        e2[r] = __ffma2_rn(m2x[r][2 * q + 1], c23, e2[r]);
-                    }
-                }
-                float e[RT];
-#pragma unroll
-                for (int r = 0; r < RT; ++r) e[r] = __fadd_rn(e2[r].x, e2[r].y);
-#pragma unroll
-                for (int r = 0; r < RT; ++r) {
-                    g2[r] = fminf(g2[r], fmaxf(g1[r], e[r]));
-                    j1[r] = (e[r] < g1[r]) ? j : j1[r];
-                    g1[r] = fminf(g1[r], e[r]);
-                }
-            }
-#pragma unroll
-            for (int r = 0; r < RT; ++r) {
-                const long long row = base + r;
-                const bool valid = row < hi;
-                const float xn2 = xnorm2_up_m2x<NP>(m2x[r]);
-                const float xn = __fsqrt_ru(xn2);
-                int lab = 0;
-                float dv = 0.f;
-                if (valid) {
-                    if (certified(g1[r], g2[r], xn2, xn, cc, gB, gp2)) {
-                        lab = j1[r];
-                        dv = d32_m2x<NP>(m2x[r], sm.Ccur + (size_t)lab * NP);
-                    } else {
-                        resc++;
-                        dv = d32_m2x<NP>(m2x[r], sm.Ccur);
-                        for (int j = 1; j < k; ++j) {
-                            const float dj = d32_m2x<NP>(m2x[r], sm.Ccur + (size_t)j * NP);
-                            if (dj < dv) { dv = dj; lab = j; }
-                        }
-                    }
-                    acc_obj(facc, dv, gf, inex);
-                }
-                if (mode == 1) {
-                    if (valid) {
-                        lab_prev[row] = lab;
-                        sm.labs[row - lo] = (unsigned short)lab;
-                        atomicAdd(&sm.lcnt[lab], 1);
-                    }
-                } else if (mode == 2) {
-                    // Move rows whose label changed between clusters.  Many
-                    // movers: each lane moves its own row.  Few movers (later
-                    // iterations): the warp moves them one at a time, lanes
-                    // over dimensions, so the warp does not walk the move path
-                    // with one or two lanes active.
-                    const bool moved = valid && oldlab[r] != lab;
-                    const unsigned mv = __ballot_sync(0xffffffffu, moved);
-                    if (__popc(mv) > 8) {
-                        if (moved) {
-                            // the row is in registers (x = -m2x / 2, exact)
-                            ok &= move_row_lane(m2x[r], oldlab[r], lab, inex);
-                            lab_prev[row] = lab;
-                        }
-                    } else {
-                        unsigned rem = mv;
-                        while (rem) {
-                            const int src = __ffs(rem) - 1;
-                            rem &= rem - 1u;
-                            const long long srow = __shfl_sync(0xffffffffu, row, src);
-                            const int snew = __shfl_sync(0xffffffffu, lab, src);
-                            const int sold = __shfl_sync(0xffffffffu, oldlab[r], src);
-                            if (lane == src) {
-                                red_s32(owner_count(snew), 1);
-                                red_s32(owner_count(sold), -1);
-                                lab_prev[srow] = snew;
-                            }
-                            const float* xr = S + srow * NP;
-                            for (int d = lane; d < n; d += 32) {
-                                __int128 v;
-                                ok &= fixed_of(xr[d], g.gx, inex, v);
-                                add_words(owner_words(snew, d), v);
-                                add_words(owner_words(sold, d), -v);
-                            }
-                        }
-                    }
-                }
-            }
+        for (long long t0 = lo; t0 < hi;) {                   // block-uniform
+            const int R = trip_rows(hi - t0);
+            const long long t1 = t0 + (long long)TPB * R;
+            assign_trip<RT>(R, t0, t1, trip_rows(hi - t1), lo, hi, mode, cc, ty);
+            t0 = t1;
         }
+        unsigned __int128& facc = ty.f;
+        unsigned int &inex = ty.inex, &resc = ty.resc;
+        bool& ok = ty.ok;
         if (mode == 1) {
             if (tracer()) atomicAdd(&a.glob->trace[15], (unsigned long long)(clock64() - t_loop));
             ok &= bucket_sums(lo, hi, inex);
@@ -794,11 +835,11 @@ struct Worker {
     }
 
     __device__ void load_row(long long i, float (&x)[NP]) const {
-        const float4* p = reinterpret_cast<const float4*>(S + i * NP);
+        float4 v[NP / 4];
+        load_chunks<0, NP>(i, v);
 #pragma unroll
         for (int q = 0; q < NP / 4; ++q) {
-            const float4 v = p[q];
-            x[4 * q] = v.x; x[4 * q + 1] = v.y; x[4 * q + 2] = v.z; x[4 * q + 3] = v.w;
+            x[4 * q] = v[q].x; x[4 * q + 1] = v[q].y; x[4 * q + 2] = v[q].z; x[4 * q + 3] = v[q].w;
         }
     }
 
@@ -957,7 +998,7 @@ struct Worker {
                     row = 0;
                 }
                 float* cb = candbuf(cpar, wid);
-                for (int d = lane; d < NP; d += 32) cb[d] = S[row * NP + d];
+                for (int d = lane; d < NP; d += 32) cb[d] = S[tile_at<NP>(row, d)];
             }
         }
         __syncthreads();
@@ -992,7 +1033,7 @@ struct Worker {
         if (!any_live) {                                     // the first centroid: uniform
             const long long pick = (long long)draw_below(a.seed, k1, 0, (unsigned long long)j, (unsigned long long)s);
             count();
-            for (int d = threadIdx.x; d < NP; d += TPB) sm.Ccur[(size_t)j * NP + d] = S[pick * NP + d];
+            for (int d = threadIdx.x; d < NP; d += TPB) sm.Ccur[(size_t)j * NP + d] = S[tile_at<NP>(pick, d)];
             __syncthreads();
             for (long long i = w0 + lane; i < w1; i += 32) {
                 float x[NP];
@@ -1025,7 +1066,7 @@ struct Worker {
                         const long long pick = (long long)draw_below(a.seed, k1, 0, (unsigned long long)j,
                                                                      (unsigned long long)s);
                         count();
-                        for (int d = threadIdx.x; d < NP; d += TPB) sm.Ccur[(size_t)j * NP + d] = S[pick * NP + d];
+                        for (int d = threadIdx.x; d < NP; d += TPB) sm.Ccur[(size_t)j * NP + d] = S[tile_at<NP>(pick, d)];
                     }
                     break;
                 }
@@ -1050,8 +1091,7 @@ struct Worker {
             auto fetch = [&](long long i) {
                 if (i < w1) {
                     d2n = dcur[i];
-#pragma unroll
-                    for (int q = 0; q < PF / 4; ++q) xn[q] = reinterpret_cast<const float4*>(S + i * NP)[q];
+                    load_chunks<0, PF>(i, xn);
                 }
             };
 #pragma unroll
@@ -1065,7 +1105,7 @@ struct Worker {
                 for (int q = 0; q < PF / 4; ++q) x[q] = xn[q];
                 const float d2 = d2n;
                 fetch(i + 32);
-                const float4* rest = reinterpret_cast<const float4*>(S + (valid ? i : w0) * NP);
+                const float* rest = S + tile_at<NP>(valid ? i : w0, 0);
                 float4 v[2][H / 4];                          // NP = 64: the chunk in hand and the next one
                 float acc[3] = {0.f, 0.f, 0.f};
                 auto add = [&](int l, const float4& xv, int q) {
@@ -1087,7 +1127,8 @@ struct Worker {
                     }
                     if (PF < NP && h + 1 < NP / H)
 #pragma unroll
-                        for (int q = 0; q < H / 4; ++q) v[(h + 1) & 1][q] = rest[(h + 1) * (H / 4) + q];
+                        for (int c = 0; c < H / 8; ++c)
+                            ld8(rest + ((h + 1) * (H / 8) + c) * 32, v[(h + 1) & 1][2 * c], v[(h + 1) & 1][2 * c + 1]);
 #pragma unroll
                     for (int l = 0; l < 3; ++l)
                         if (go[l])
