@@ -404,18 +404,30 @@ void set_fullpass_impl(int impl) { g_fullpass_impl.store(impl); }
 int last_fullpass_impl() { return g_last_impl; }
 int fullpass_impl_setting() { return g_fullpass_impl.load(); }
 // By shape: the FP32-ALU pass costs about k NP / 2 packed FMAs per row, the
-// tensor-core pass a fixed epilogue per row and centroid column, so the
-// tensor cores win once the contraction per row is large.  Measured on GB300
-// (10^6 x 16 and 4 10^6 x 32): the lean pass (NP <= 32) wins from NP k = 800
-// (n = 16, k = 50: 55 against 67 us; n = 32, k = 25: 201 against 264 us) and
-// loses at NP k <= 400 (n = 16, k = 25: 49 against 43 us); the NP = 64 pass
-// from NP k > 1600.
-bool fullpass_prefers_tensor(int np, int k) { return (long long)np * k > (np <= 32 ? 512 : 1600); }
+// tensor-core pass mostly a fixed amount per row (split, direct form,
+// barriers) and little per column, and it starts slower.  Measured on GB300,
+// ALU against tensor cores, us (kernel, rows not in L2):
+//   10^6 x 2,  k = 5:  21 / 33      10^6 x 8,  k = 10: 27 / 33
+//   10^6 x 16, k = 25: 44 / 36      10^6 x 8,  k = 100: 81 / 46
+//   4 10^6 x 32, k = 10: 177 / 136  4 10^6 x 32, k = 50: 421 / 173
+//   10^6 x 64, k = 10: 111 / 70     10^7 x 64, k = 100: 4137 / 857
+// so the line lies at NP k = 256.  Widths that are no multiple of 4 come by
+// 1-D copies and are read word by word from shared memory, which moves it:
+//   10^6 x 63, k = 7: 109 / 124     1.5 10^6 x 21, k = 33: 115 / 95
+// Up to 131,072 rows (about a tile per warpgroup) the start dominates and the
+// two are within 2 us of each other below NP k = 512 (NP <= 32) or 1600:
+//   5 10^4 x 16, k = 25: 15 / 15    5 10^4 x 16, k = 50: 19 / 15
+bool fullpass_prefers_tensor(long long m, int n, int np, int k) {
+    const long long w = (long long)np * k;
+    if (n % 4 != 0) return m > 131072 && w >= 768;
+    return m > 131072 ? w >= 256 : w > (np <= 32 ? 512 : 1600);
+}
 cudaError_t launch_fullpass(int np, const float* X, long long m, int n, const float* C, int k,
                             const double* sel_f, int W, int* labels, Globals* g, float gB, float gp2,
                             int incumbent, int sms, cudaStream_t st) {
     int impl = g_fullpass_impl.load();
-    if (impl == 0) impl = fullpass_prefers_tensor(np, k) ? 2 : 1;
+    if (impl == 0) impl = fullpass_prefers_tensor(m, n, np, k) ? 2 : 1;
+    else if (n % 4 != 0) impl = 1;                 // asked for by number: n % 4 == 0 only, as documented
     if (impl == 2) {
         const cudaError_t e = launch_tcx_fullpass(np, X, m, n, C, k, sel_f, W, labels, g, gB, gp2, incumbent, sms, st);
         if (e != cudaErrorNotSupported) {

@@ -4,6 +4,8 @@
 #pragma once
 #include <cstdint>
 
+#include <cuda_bf16.h>
+
 #include "bm_device.cuh"
 
 namespace bm {
@@ -63,6 +65,15 @@ __device__ __forceinline__ bool wait(unsigned long long* b, unsigned parity, vol
     return false;
 }
 
+// The same wait by every lane of a warp (no lane has to pass the outcome on);
+// true for all lanes or for none.
+__device__ __forceinline__ bool wait_warp(unsigned long long* b, unsigned parity, volatile int* abort, Globals* g,
+                                          WaitLimit lim) {
+    bool ok = try_wait(b, parity);
+    if (!ok) ok = wait(b, parity, abort, g, lim);
+    return __all_sync(0xffffffffu, ok);
+}
+
 // 1-D bulk copy global -> shared (addresses and size multiples of 16 bytes).
 __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, unsigned bytes, unsigned long long* b) {
     asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
@@ -92,12 +103,9 @@ __device__ __forceinline__ unsigned long long desc_sw128(unsigned addr) {
     return d;
 }
 // Instruction descriptors: FP32 accumulate, A and B K-major, M x N.
-//   kind::f16 with BF16 operands (format 1); kind::tf32 (format 2).
+// kind::f16 with BF16 operands (format 1).
 __host__ __device__ constexpr unsigned idesc_bf16(int M, int N) {
     return (1u << 4) | (1u << 7) | (1u << 10) | ((unsigned)(N >> 3) << 17) | ((unsigned)(M >> 4) << 24);
-}
-__host__ __device__ constexpr unsigned idesc_tf32(int M, int N) {
-    return (1u << 4) | (2u << 7) | (2u << 10) | ((unsigned)(N >> 3) << 17) | ((unsigned)(M >> 4) << 24);
 }
 
 __device__ __forceinline__ void mma_bf16(unsigned tmem_d, unsigned long long adesc, unsigned long long bdesc,
@@ -105,14 +113,6 @@ __device__ __forceinline__ void mma_bf16(unsigned tmem_d, unsigned long long ade
     asm volatile(
         "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
         " tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}" ::"r"(tmem_d),
-        "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-__device__ __forceinline__ void mma_tf32(unsigned tmem_d, unsigned long long adesc, unsigned long long bdesc,
-                                         unsigned idesc, unsigned accumulate) {
-    asm volatile(
-        "{\n .reg .pred p;\n setp.ne.b32 p, %4, 0;\n"
-        " tcgen05.mma.cta_group::1.kind::tf32 [%0], %1, %2, %3, p;\n}" ::"r"(tmem_d),
         "l"(adesc), "l"(bdesc), "r"(idesc), "r"(accumulate)
         : "memory");
 }
@@ -223,11 +223,88 @@ __device__ __forceinline__ unsigned le_mask16(const unsigned (&va)[16], const fl
     return PART ? mk & ((1u << nv) - 1u) : mk;
 }
 
-// Round to TF32 (10 explicit mantissa bits), to nearest, ties away from zero.
-__device__ __forceinline__ float to_tf32(float x) {
-    unsigned r;
-    asm("cvt.rna.tf32.f32 %0, %1;" : "=r"(r) : "f"(x));
-    return __uint_as_float(r);
+// 32 lanes x 32 columns of 32-bit tensor-memory cells -> 32 registers per
+// thread, waited for (the wait takes the registers as operands, so that no use
+// of them can be scheduled before it).
+__device__ __forceinline__ void wait_ld32(unsigned (&r)[32]) {
+    asm volatile("tcgen05.wait::ld.sync.aligned;"
+                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
+                   "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]),
+                   "+r"(r[15]), "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]),
+                   "+r"(r[22]), "+r"(r[23]), "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]),
+                   "+r"(r[29]), "+r"(r[30]), "+r"(r[31])
+                 :
+                 : "memory");
+}
+__device__ __forceinline__ void ld32(unsigned taddr, unsigned (&r)[32]) {
+    asm volatile("tcgen05.ld.sync.aligned.32x32b.x32.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+                   "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]),
+                   "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]),
+                   "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]),
+                   "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
+                 : "r"(taddr));
+    wait_ld32(r);
+}
+// The same, with the least of the 32 values (as FP32) taken on the way.
+__device__ __forceinline__ void ld32_min(unsigned taddr, unsigned (&r)[32], float& mn) {
+    unsigned u;
+    asm volatile("tcgen05.ld.red.sync.aligned.32x32b.x32.min.f32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, %32, [%33];"
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
+                   "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]),
+                   "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]),
+                   "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]),
+                   "=r"(r[29]), "=r"(r[30]), "=r"(r[31]), "=r"(u)
+                 : "r"(taddr));
+    wait_ld32(r);
+    asm volatile("" : "+r"(u));                    // not before the wait either
+    mn = __uint_as_float(u);
+}
+// 32 floats of shared memory (16-byte aligned) into 32 columns of every lane
+// of the warp (pair with wait_st).
+__device__ __forceinline__ void st32_shared(unsigned taddr, const float* p) {
+    unsigned r[32];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+        const uint4 v = *reinterpret_cast<const uint4*>(p + 4 * q);
+        r[4 * q] = v.x; r[4 * q + 1] = v.y; r[4 * q + 2] = v.z; r[4 * q + 3] = v.w;
+    }
+    asm volatile("tcgen05.st.sync.aligned.32x32b.x32.b32 [%32], {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, %16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31};" ::"r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]),
+                 "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(r[16]),
+                 "r"(r[17]), "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]), "r"(r[24]),
+                 "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31]), "r"(taddr)
+                 : "memory");
+}
+__device__ __forceinline__ void wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
+
+// Bit 31 - i set where the i-th of 32 values is below L: v - L is exact in
+// sign (gradual underflow), and a funnel shift moves the sign bit in.
+__device__ __forceinline__ unsigned below_mask32(const unsigned (&va)[32], float L) {
+    unsigned mk = 0;
+    const float2 mL = make_float2(-L, -L);
+#pragma unroll
+    for (int i = 0; i < 32; i += 2) {
+        const float2 d = __fadd2_rn(make_float2(__uint_as_float(va[i]), __uint_as_float(va[i + 1])), mL);
+        mk = __funnelshift_l(__float_as_uint(d.x), mk, 1);
+        mk = __funnelshift_l(__float_as_uint(d.y), mk, 1);
+    }
+    return mk;
+}
+
+// Eight values as BF16 pairs h = bf16(v) and l = bf16(v - h) (v - h is exact).
+__device__ __forceinline__ void split_bf16(const float (&v)[8], uint4& h, uint4& l) {
+    unsigned hw[4], lw[4];
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const __nv_bfloat162 a = __floats2bfloat162_rn(v[2 * i], v[2 * i + 1]);
+        hw[i] = *reinterpret_cast<const unsigned*>(&a);
+        const float2 f = make_float2(__uint_as_float(hw[i] << 16), __uint_as_float(hw[i] & 0xffff0000u));
+        const float2 r = __ffma2_rn(make_float2(-1.f, -1.f), f, make_float2(v[2 * i], v[2 * i + 1]));
+        const __nv_bfloat162 b = __floats2bfloat162_rn(r.x, r.y);
+        lw[i] = *reinterpret_cast<const unsigned*>(&b);
+    }
+    h = make_uint4(hw[0], hw[1], hw[2], hw[3]);
+    l = make_uint4(lw[0], lw[1], lw[2], lw[3]);
 }
 
 }  // namespace tc
