@@ -491,11 +491,13 @@ int32_t bm_get_big_clusters(void);
 /* How samples are drawn without replacement (Sec. 4.1: a uniform sample of
  * s distinct points, here the first s distinct values of the job's counter
  * stream of bounded draws, in order of first occurrence).  impl 0 (default):
- * a shared-memory bitmap of the m indices where it fits (m up to about
- * 1.37e6: the bitmap and the per-chunk hash table within 200 KB), else
- * per-job open-addressing tables in device memory; impl 1: always the
- * tables.
- * Both give identical samples.  Other values: BM_EINVAL.  Process-wide,
+ * where the largest sample has at least 4096 rows and at most m / 2, many CTAs
+ * per sample on open-addressing tables in device memory; else, and for the
+ * samples a fit draws ahead while its workers run, one CTA per sample with a
+ * shared-memory bitmap of the m indices where it fits (m up to about 1.37e6:
+ * the bitmap and the per-chunk hash table within 200 KB); else one CTA per
+ * sample on the tables; impl 1: always the last.
+ * All give identical samples.  Other values: BM_EINVAL.  Process-wide,
  * read when each sampling launch is prepared. */
 bm_status bm_set_sampler_impl(int32_t impl);
 int32_t bm_get_sampler_impl(void);

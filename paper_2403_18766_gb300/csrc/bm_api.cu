@@ -38,7 +38,7 @@ cudaError_t launch_fullpass(int np, const float* X, long long m, int n, const fl
 cudaError_t launch_prepass(const float* v, long long count, Globals* g, const float* C, int k, int n, int np,
                            float* Cp, int sms, cudaStream_t st);
 cudaError_t launch_pad(const float* src, long long rows, int n, int np, float* dst, cudaStream_t st);
-cudaError_t launch_unpad(const float* src, long long rows, int n, int np, float* dst, int tiles, cudaStream_t st);
+cudaError_t launch_unpad(const float* src, long long rows, int n, int np, float* dst, cudaStream_t st);
 cudaError_t launch_select_unpad(const float* Cw, const double* sel_f, int W, int k, int n, int np,
                                 float* dst, cudaStream_t st);
 cudaError_t launch_init_state(double* fhat, int W, unsigned char* deg, long long kdeg, Globals* g,
@@ -254,7 +254,10 @@ struct bm_fit_ctx {
     int rounds_planned = 0x7fffffff;        // rounds the caller intends to run (T)
     cudaStream_t sst = nullptr;             // sampling stream (draws the next round ahead)
     cudaEvent_t ev_sdone = nullptr;
-    unsigned int gen = 1;                   // next sampler-table generation
+    unsigned int gen = 1;                   // next sampler-table generation (a CTA per job)
+    unsigned int wgen = 0;                  // last generation of the launches with many CTAs per job
+    int table_fmt[2] = {0, 0};              // slot format of each half's tables (0: not cleared yet)
+    int* wcnt = nullptr;                    // first-occurrence counts and flags of those launches
     float* S = nullptr; long long* idx = nullptr; unsigned int* draws = nullptr;
     unsigned long long* table = nullptr; int* job_s = nullptr; float* D2 = nullptr; int* lab = nullptr;
     float* Cw = nullptr; float* Cw_cta = nullptr; unsigned char* deg = nullptr;
@@ -336,8 +339,28 @@ WorkerArgs make_args(const bm_fit_ctx* c, int mode, int parity = 0) {
     return a;
 }
 
-SampleArgs make_sample_args(bm_fit_ctx* c, int mode, int jobs, int parity = 0) {
-    SampleArgs a;
+// Smallest largest sample drawn by many CTAs per job (below, one launch of a
+// CTA per job is as quick: fit of 10^4 x 2 with samples up to 2000).
+constexpr long long kWideMin = 4096;
+int wide_chunks(const bm_fit_ctx* c) { return (int)((c->Tcap + kWideDraws - 1) / kWideDraws); }
+// Many CTAs per job: a table that half fills at most (2 s <= m keeps the
+// draws few), draw indices of 20 bits, jobs as a grid dimension.
+bool wide_sampling(const bm_fit_ctx* c, int jobs) {
+    return !g_sample_tables.load() && c->s_cap >= kWideMin && 2 * c->s_cap <= c->m &&
+           c->Tcap < (1ll << kWideTBits) && jobs <= 65535;
+}
+
+// Arguments of a sampling launch on stream `st`.  The launch's half of the
+// tables is cleared there first when it has not been used in this launch's
+// slot format yet (or its generations have run out).
+// `ahead`: the launch runs beside a worker launch, on the SMs that leaves
+// free.  There a job per CTA is the better form while its bitmap fits: it
+// touches memory for the rows alone, where the tables of many jobs at once
+// (clearing them included) take bandwidth and the few free SMs are busy either
+// way (fit of 10^6 x 16, k = 25, 16 workers, 4 rounds: 7.4 ms against 8.1 ms
+// with many CTAs per job in every round).
+bm_status make_sample_args(bm_fit_ctx* c, int mode, int jobs, int parity, bool ahead, cudaStream_t st,
+                           SampleArgs& a) {
     memset(&a, 0, sizeof a);
     a.X = c->X; a.m = c->m; a.n = c->n; a.mode = mode; a.seed = c->seed;
     a.W = c->pol.workers; a.P = c->pol.passes;
@@ -354,15 +377,32 @@ SampleArgs make_sample_args(bm_fit_ctx* c, int mode, int jobs, int parity = 0) {
     a.idx_stride = c->s_cap; a.idx = c->idx + J * a.idx_stride;
     a.draws_stride = c->Tcap; a.draws = c->draws + J * a.draws_stride; a.Tcap = c->Tcap;
     a.H = c->H; a.table_stride = c->H; a.table = c->table + J * a.table_stride;
-    a.gen_base = c->gen;
-    c->gen += (unsigned int)jobs;
+    a.chunks = wide_chunks(c);
+    a.wcnt = c->wcnt + J * a.chunks * (1 + kWideDraws / 32);
+    a.job_s = c->job_s + J; a.glob = c->glob;
     // shared-memory bitmap of the m values when it fits in one CTA
     const long long words = (c->m + 31) / 32;
     const size_t sb = sample_smem_bytes((int)std::min<long long>(words, 1 << 30));
-    if (mode != kSampleGather && !g_sample_tables.load() && words <= (1 << 30) && sb <= 200 * 1024)
-        a.bitmap_words = (int)words;
-    a.job_s = c->job_s + J; a.glob = c->glob;
-    return a;
+    const bool bitmap = !g_sample_tables.load() && words <= (1 << 30) && sb <= 200 * 1024;
+    a.wide = wide_sampling(c, jobs) && !(ahead && bitmap);
+    if (!a.wide && bitmap) a.bitmap_words = (int)words;
+    if (a.bitmap_words > 0) return BM_OK;                 // no table
+    if (a.wide) {
+        if (c->wgen == kWideGens) {                       // generations start again: both halves are stale
+            c->wgen = 0;
+            c->table_fmt[0] = c->table_fmt[1] = 0;
+        }
+        a.wgen = ++c->wgen;
+    } else {
+        a.gen_base = c->gen;
+        c->gen += (unsigned int)jobs;
+    }
+    const int fmt = a.wide ? 2 : 1;
+    if (c->table_fmt[parity] != fmt) {
+        CU(cudaMemsetAsync(c->table + (long long)parity * c->jobs * c->H, 0, (size_t)c->jobs * c->H * 8, st));
+        c->table_fmt[parity] = fmt;
+    }
+    return BM_OK;
 }
 
 cudaEvent_t take_event(bm_fit_ctx* c) {
@@ -439,6 +479,7 @@ size_t workspace_bytes(const bm_fit_ctx* c, int W) {
     take((size_t)J * c->s_cap * 8);
     take((size_t)J * c->Tcap * 4);
     take((size_t)J * c->H * 8);
+    take((size_t)J * wide_chunks(c) * (1 + kWideDraws / 32) * 4);
     take((size_t)J * 4);
     take((size_t)W * 4 * c->s_cap * 4);
     take((size_t)W * c->s_cap * 4);
@@ -464,6 +505,7 @@ bm_status alloc_workspace(bm_fit_ctx* c, int W) {
     const size_t o_idx = take((size_t)J * c->s_cap * 8);
     const size_t o_draws = take((size_t)J * c->Tcap * 4);
     const size_t o_tab = take((size_t)J * c->H * 8);
+    const size_t o_wc = take((size_t)J * wide_chunks(c) * (1 + kWideDraws / 32) * 4);
     const size_t o_js = take((size_t)J * 4);
     const size_t o_D2 = take((size_t)W * 4 * c->s_cap * 4);
     const size_t o_lab = take((size_t)W * c->s_cap * 4);
@@ -494,6 +536,7 @@ bm_status alloc_workspace(bm_fit_ctx* c, int W) {
     c->glob = (Globals*)(b + o_glob);
     c->S = (float*)(b + o_S); c->idx = (long long*)(b + o_idx); c->draws = (unsigned int*)(b + o_draws);
     c->table = (unsigned long long*)(b + o_tab); c->job_s = (int*)(b + o_js);
+    c->wcnt = (int*)(b + o_wc);
     c->D2 = (float*)(b + o_D2); c->kx = (long long*)(b + o_kx); c->lab = (int*)(b + o_lab); c->Cw = (float*)(b + o_Cw); c->Cw_cta = (float*)(b + o_Cwc);
     c->deg = (unsigned char*)(b + o_deg); c->fhat = (double*)(b + o_fhat); c->f_final = (double*)(b + o_ff);
     c->L_buf = (long long*)(b + o_L); c->timer = (unsigned long long*)(b + o_t);
@@ -504,7 +547,6 @@ bm_status alloc_workspace(bm_fit_ctx* c, int W) {
     }
     CU(cudaMemsetAsync(c->glob, 0, sizeof(Globals), c->st));
     CU(cudaMemsetAsync(c->Cw, 0, (size_t)W * k * np * 4, c->st));
-    CU(cudaMemsetAsync(c->table, 0, (size_t)J * c->H * 8, c->st));
     CU(cudaMemsetAsync(c->job_s, 0, (size_t)J * 4, c->st));
     return BM_OK;
 }
@@ -704,9 +746,10 @@ bm_status round_samples(bm_fit_ctx* c, int r0) {
         CU(cudaStreamWaitEvent(c->st, c->ev_sdone, 0));           // drawn ahead on the sampling stream
     } else {
         if (c->prefetched >= 0) CU(cudaStreamWaitEvent(c->st, c->ev_sdone, 0));
-        SampleArgs sa = make_sample_args(c, kSampleRound, c->jobs, parity);
-        sa.rnd = r0;
         const size_t sp_s = span_begin(c, 2);
+        SampleArgs sa;
+        if ((s = make_sample_args(c, kSampleRound, c->jobs, parity, false, c->st, sa))) return s;
+        sa.rnd = r0;
         CU(launch_sample(c->np, sa, (c->w_hi - c->w_lo) * (c->pol.passes + 1), c->st));
         span_end(c, sp_s);
         c->n_kernels++;
@@ -722,9 +765,10 @@ bm_status round_samples(bm_fit_ctx* c, int r0) {
 bm_status round_prefetch(bm_fit_ctx* c, int r0) {
     if (r0 + 1 < c->rounds_planned && c->pol.exploit == 0) {
         CU(cudaStreamWaitEvent(c->sst, c->ev_fork, 0));
-        SampleArgs sa = make_sample_args(c, kSampleRound, c->jobs, (r0 + 1) & 1);
-        sa.rnd = r0 + 1;
         const size_t sp_s = span_begin(c, 2, c->sst);
+        SampleArgs sa;
+        if (const bm_status s = make_sample_args(c, kSampleRound, c->jobs, (r0 + 1) & 1, true, c->sst, sa)) return s;
+        sa.rnd = r0 + 1;
         CU(launch_sample(c->np, sa, (c->w_hi - c->w_lo) * (c->pol.passes + 1), c->sst));
         span_end(c, sp_s);
         CU(cudaEventRecord(c->ev_sdone, c->sst));
@@ -1133,7 +1177,9 @@ bm_status bm_fit_recheck(bm_fit_ctx* c, int64_t s_opt, double* f_out_host) {
         c->prefetched = -1;
     }
     const size_t sp = span_begin(c, 0);
-    SampleArgs sa = make_sample_args(c, kSampleFinal, 1);
+    SampleArgs sa;
+    bm_status s;
+    if ((s = make_sample_args(c, kSampleFinal, 1, 0, false, c->st, sa))) return s;
     sa.step_s = s_opt;
     CU(launch_sample(c->np, sa, 1, c->st));
     WorkerArgs a = make_args(c, kModeFinalEval);
@@ -1144,7 +1190,6 @@ bm_status bm_fit_recheck(bm_fit_ctx* c, int64_t s_opt, double* f_out_host) {
     CU(cudaMemcpyAsync(f_out_host, c->f_final + c->w_lo, (size_t)(c->w_hi - c->w_lo) * 8, cudaMemcpyDeviceToHost,
                        c->st));
     Globals h;
-    bm_status s;
     if ((s = read_globals(c, &h))) return s;
     return status_from_flags(h);
 }
@@ -1154,7 +1199,7 @@ bm_status bm_fit_worker_centroids(bm_fit_ctx* c, int32_t w, float* C_out_dev) {
     if (w < c->w_lo || w >= c->w_hi) return fail(BM_EINVAL, "worker %d not in [%d, %d)", w, c->w_lo, c->w_hi);
     bm_status s = check_ptr(C_out_dev, "C_out_dev");
     if (s) return s;
-    CU(launch_unpad(c->Cw + (size_t)w * c->k * c->np, c->k, c->n, c->np, C_out_dev, 0, c->st));
+    CU(launch_unpad(c->Cw + (size_t)w * c->k * c->np, c->k, c->n, c->np, C_out_dev, c->st));
     CU(cudaStreamSynchronize(c->st));
     return BM_OK;
 }
@@ -1180,7 +1225,8 @@ static bm_status fit_finish(bm_fit_ctx* c, float* C_out_dev, int32_t* labels_out
         c->prefetched = -1;
     }
     const size_t sp = span_begin(c, 0);
-    SampleArgs sa = make_sample_args(c, kSampleFinal, 1);
+    SampleArgs sa;
+    if ((s = make_sample_args(c, kSampleFinal, 1, 0, false, c->st, sa))) return s;
     CU(launch_sample(c->np, sa, 1, c->st));
     CU(launch_worker(c->np, a, c->pol.workers, c->st));
     c->n_kernels += 2;
@@ -1494,9 +1540,10 @@ bm_status bigmeans_fit_host(const float* X_host, int64_t m, int32_t n, int32_t k
 }
 
 // ------------------------------------------------------------- step calls
-// A one-worker context with explicit sizes, used by the step entry points.
-static bm_status step_ctx(bm_fit_ctx* c, const float* X, long long m, int n, int k, long long s_cap,
-                          unsigned long long seed, void* stream) {
+// A one-worker context with explicit sizes, used by the step entry points
+// (step_plan: sizes and their checks alone).
+static bm_status step_plan(bm_fit_ctx* c, const float* X, long long m, int n, int k, long long s_cap,
+                           unsigned long long seed, void* stream) {
     c->st = (cudaStream_t)stream;
     c->X = X; c->m = m; c->n = n; c->k = k; c->np = padded_dim(n);
     c->pol = bm_sample_policy{};
@@ -1515,7 +1562,12 @@ static bm_status step_ctx(bm_fit_ctx* c, const float* X, long long m, int n, int
     c->H = next_pow2(2 * c->Tcap);
     c->L_cap = 1;
     cert_constants(c->np, c->gB, c->gp2);
-    return alloc_workspace(c, 1);
+    return BM_OK;
+}
+static bm_status step_ctx(bm_fit_ctx* c, const float* X, long long m, int n, int k, long long s_cap,
+                          unsigned long long seed, void* stream) {
+    const bm_status s = step_plan(c, X, m, n, k, s_cap, seed, stream);
+    return s ? s : alloc_workspace(c, 1);
 }
 
 struct CtxGuard {
@@ -1534,7 +1586,8 @@ bm_status bm_sample(uint64_t seed, int32_t purpose, int32_t worker, int32_t roun
     CtxGuard guard{c};
     bm_status st = step_ctx(c, nullptr, m, 1, 1, s, seed, stream);
     if (st) return st;
-    SampleArgs a = make_sample_args(c, kSampleStep, 1);
+    SampleArgs a;
+    if ((st = make_sample_args(c, kSampleStep, 1, 0, false, c->st, a))) return st;
     a.idx = reinterpret_cast<long long*>(idx_out_dev); a.idx_stride = 0;
     a.step_s = s; a.purpose = purpose; a.worker = worker; a.rnd = round; a.pss = pass;
     CU(launch_sample(c->np, a, 1, c->st));
@@ -1552,13 +1605,15 @@ bm_status bm_gather(const float* X_dev, int64_t m, int32_t n, const int64_t* idx
     if (!X_dev || !idx_dev || !S_out_dev) return fail(BM_EINVAL, "NULL pointer");
     bm_fit_ctx* c = new bm_fit_ctx();
     CtxGuard guard{c};
-    if ((st = step_ctx(c, X_dev, m, n, 1, s, 0, stream))) return st;
-    SampleArgs a = make_sample_args(c, kSampleGather, 1);
-    a.idx = const_cast<long long*>(reinterpret_cast<const long long*>(idx_dev));
-    a.idx_stride = 0;
-    a.step_s = s;
-    CU(launch_sample(c->np, a, 1, c->st));
-    CU(launch_unpad(c->S, s, n, c->np, S_out_dev, 1, c->st));
+    if ((st = step_plan(c, X_dev, m, n, 1, s, 0, stream))) return st;
+    if (lib_alloc(&c->base, sizeof(Globals), c->st) != cudaSuccess) {
+        c->base = nullptr;
+        cudaGetLastError();
+        return fail(BM_ENOMEM, "workspace of %zu bytes", sizeof(Globals));
+    }
+    c->glob = (Globals*)c->base;
+    CU(cudaMemsetAsync(c->glob, 0, sizeof(Globals), c->st));
+    CU(launch_gather(X_dev, m, n, reinterpret_cast<const long long*>(idx_dev), s, S_out_dev, c->glob, c->st));
     Globals h;
     if ((st = read_globals(c, &h))) return st;
     return status_from_flags(h);
@@ -1586,7 +1641,7 @@ bm_status bm_kmeanspp(const float* S_dev, int64_t s, int32_t n, float* C_inout_d
     WorkerArgs a = make_args(c, kModeStepKpp);
     a.trials = trials; a.step_s = s; a.step_worker = worker; a.step_round = round; a.step_pass = pass;
     CU(launch_worker(c->np, a, 1, c->st));
-    CU(launch_unpad(c->Cw, k, n, c->np, C_inout_dev, 0, c->st));
+    CU(launch_unpad(c->Cw, k, n, c->np, C_inout_dev, c->st));
     Globals h;
     if ((st = read_globals(c, &h))) return st;
     return status_from_flags(h);
@@ -1610,7 +1665,7 @@ bm_status bm_lloyd(const float* S_dev, int64_t s, int32_t n, float* C_inout_dev,
     a.step_f = c->f_final; a.step_iters = (int*)c->L_buf;
     a.step_empty = empty_out_dev ? empty_out_dev : c->deg;
     CU(launch_worker(c->np, a, 1, c->st));
-    CU(launch_unpad(c->Cw, k, n, c->np, C_inout_dev, 0, c->st));
+    CU(launch_unpad(c->Cw, k, n, c->np, C_inout_dev, c->st));
     double f = 0;
     int it = 0;
     CU(cudaMemcpyAsync(&f, c->f_final, 8, cudaMemcpyDeviceToHost, c->st));

@@ -320,7 +320,7 @@ fullpass_kernel(const float* __restrict__ X, long long m, int n, const float* __
 
 // ----------------------------------------------------------- small kernels
 // Copy rows of width n into a sample's tiles of padded rows (tile_at), or
-// back from padded rows (tiles or row-major).
+// rows of width n out of padded row-major rows.
 __global__ void pad_rows_kernel(const float* __restrict__ src, long long rows, int n, int np,
                                 float* __restrict__ dst) {
     const long long total = rows * np;
@@ -332,13 +332,13 @@ __global__ void pad_rows_kernel(const float* __restrict__ src, long long rows, i
     }
 }
 __global__ void unpad_rows_kernel(const float* __restrict__ src, long long rows, int n, int np,
-                                  float* __restrict__ dst, int tiles) {
+                                  float* __restrict__ dst) {
     const long long total = rows * n;
     for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < total;
          e += (long long)gridDim.x * blockDim.x) {
         const long long i = e / n;
         const int d = (int)(e % n);
-        dst[e] = src[tiles ? tile_at(np, i, d) : i * np + d];
+        dst[e] = src[i * np + d];
     }
 }
 // Select the centroids of argmin sel_f (lowest index) and unpad them.
@@ -462,11 +462,11 @@ cudaError_t launch_pad(const float* src, long long rows, int n, int np, float* d
     pad_rows_kernel<<<grid, 256, 0, st>>>(src, rows, n, np, dst);
     return cudaGetLastError();
 }
-cudaError_t launch_unpad(const float* src, long long rows, int n, int np, float* dst, int tiles, cudaStream_t st) {
+cudaError_t launch_unpad(const float* src, long long rows, int n, int np, float* dst, cudaStream_t st) {
     if (rows <= 0) return cudaSuccess;
     const long long total = rows * n;
     const int grid = (int)min(4096ll, (total + 255) / 256);
-    unpad_rows_kernel<<<grid, 256, 0, st>>>(src, rows, n, np, dst, tiles);
+    unpad_rows_kernel<<<grid, 256, 0, st>>>(src, rows, n, np, dst);
     return cudaGetLastError();
 }
 cudaError_t launch_select_unpad(const float* Cw, const double* sel_f, int W, int k, int n, int np,

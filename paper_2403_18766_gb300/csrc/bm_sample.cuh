@@ -10,7 +10,6 @@ enum SampleMode : int {
     kSampleRound = 0,   // every (worker, slot) job of one round: slots 0..P-1 passes, P = eval
     kSampleFinal = 1,   // the common sample of size s_opt (one job)
     kSampleStep = 2,    // one explicit stream, indices only
-    kSampleGather = 3,  // one job, indices given in idx: gather only
 };
 
 // Sample-size policy of one round (Alg. 1 "s_w <- random size", and the
@@ -86,6 +85,12 @@ struct SampleArgs {
     unsigned int gen_base;                     // generation of job 0 (tables are never cleared)
     int bitmap_words;                          // > 0: draw with a shared-memory bitmap of the m
                                                // values ((m + 31) / 32 words) instead of the tables
+    // many CTAs per job (sample_wide_*): per job `chunks` chunks of
+    // kWideDraws draws, a count and 32 words of flags each
+    int wide;                                  // 1: draw with them instead of sample_kernel
+    unsigned int wgen;                         // generation of the launch, 1 .. kWideGens
+    int chunks;
+    int* wcnt;                                 // jobs x chunks x (1 + kWideDraws / 32)
     int* job_s;                                // out: sample size of each job
     Globals* glob;
 };
@@ -96,12 +101,20 @@ constexpr int kSampleThreads = 1024;
 // per-chunk hash table (2 per draw).
 constexpr int kSampleDraws = 2;
 constexpr int kMiniSlots = 2 * kSampleDraws * kSampleThreads;
+// Many CTAs per job: draws of a CTA; a table slot holds generation (13 bits),
+// value (31) and draw index (20).
+constexpr int kWideDraws = 1024;
+constexpr int kWideTBits = 20;
+constexpr unsigned kWideGens = 8191;
 // Items a thread of the gather has in flight at once.
 constexpr int kGatherBatch = 8;
 // Dynamic shared memory of a sampling launch.
 inline size_t sample_smem_bytes(int bitmap_words) {
     return bitmap_words > 0 ? (size_t)kMiniSlots * 8 + (((size_t)bitmap_words * 4 + 15) & ~(size_t)15) : 0;
 }
+// Rows idx[i] of X (m x n) to out (s x n); an index outside [0, m) sets kErrArgs.
+cudaError_t launch_gather(const float* X, long long m, int n, const long long* idx, long long s, float* out,
+                          Globals* g, cudaStream_t st);
 cudaError_t launch_sample(int np, const SampleArgs& a, int jobs, cudaStream_t st);
 
 }  // namespace bm
