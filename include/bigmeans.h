@@ -446,9 +446,10 @@ int32_t bm_last_fullpass_impl(void);
  *   Worker groups (default): when every worker gets a cluster of 8 CTAs and
  *   the whole launch can be resident at once (a cooperative launch), the
  *   clusters the device can hold beyond one per worker go to the workers
- *   with the most sample rows per CTA, so a large sample spans up to 8
- *   clusters (64 CTAs) that add up their exact partial sums in global memory
- *   with a barrier among the group's CTAs; rows per CTA then stay about
+ *   with the most sample rows per CTA, so a large sample spans up to 32
+ *   clusters (256 CTAs) that add up their exact partial sums in global memory
+ *   with a barrier among the group's CTAs (bm_kmeanspp and bm_lloyd: the one
+ *   worker has the device to itself); rows per CTA then stay about
  *   equal across workers.  Each such barrier is bounded (a few seconds):
  *   when one runs out the round returns BM_ETIMEOUT.
  *   Otherwise (bm_set_worker_groups(0), more workers than resident clusters,

@@ -304,7 +304,7 @@ long long sample_floats(const bm_fit_ctx* c) { return (c->s_cap + 3) / 4 * 4 * c
 // (more workers than a cooperative launch can hold clusters, or too large).
 size_t group_bytes(const bm_fit_ctx* c, int W) {
     if (W > kMaxGroupWorkers) return 0;
-    const size_t part = (size_t)W * 2 * kMaxGroup * c->k * c->np * kAccWords * 8;
+    const size_t part = (size_t)W * 3 * c->k * c->np * kAccWords * 8;
     if (part > ((size_t)256 << 20)) return 0;
     return part;
 }
@@ -469,9 +469,9 @@ size_t workspace_bytes(const bm_fit_ctx* c, int W) {
     auto take = [&](size_t bytes) { off += (bytes + 255) & ~(size_t)255; };
     if (const size_t gb = group_bytes(c, W)) {
         take(gb);
-        take((size_t)W * 2 * kMaxGroup * k * 4);
-        take((size_t)W * 2 * kMaxGroup * 4 * 8);
+        take((size_t)W * 3 * k * 4);
         take((size_t)W * 2 * 4);
+        take((size_t)W * 2 * kMaxGroup * 4 * 8);
         take((size_t)W * 2 * 4);
     }
     take(sizeof(Globals));
@@ -492,6 +492,14 @@ size_t workspace_bytes(const bm_fit_ctx* c, int W) {
     take((size_t)c->L_cap * 8);
     take(8);
     return off;
+}
+
+// Before a launch with groups: the group sums, counts, barriers and abort
+// flags (one piece of the workspace) are zero.
+cudaError_t clear_group_state(const bm_fit_ctx* c, cudaStream_t st) {
+    if (!c->xbar) return cudaSuccess;
+    const char* end = reinterpret_cast<const char*>(c->xbar) + (size_t)c->pol.workers * 2 * 4;
+    return cudaMemsetAsync(c->xpart, 0, (size_t)(end - reinterpret_cast<const char*>(c->xpart)), st);
 }
 
 bm_status alloc_workspace(bm_fit_ctx* c, int W) {
@@ -521,9 +529,9 @@ bm_status alloc_workspace(bm_fit_ctx* c, int W) {
     size_t o_xp = 0, o_xc = 0, o_xo = 0, o_xb = 0, o_xf = 0;
     if (gb) {
         o_xp = take(gb);
-        o_xc = take((size_t)W * 2 * kMaxGroup * k * 4);
-        o_xo = take((size_t)W * 2 * kMaxGroup * 4 * 8);
+        o_xc = take((size_t)W * 3 * k * 4);
         o_xb = take((size_t)W * 2 * 4);
+        o_xo = take((size_t)W * 2 * kMaxGroup * 4 * 8);
         o_xf = take((size_t)W * 2 * 4);
     }
     cudaError_t e = lib_alloc(&c->base, off, c->st);
@@ -794,7 +802,7 @@ bm_status run_round_launch(bm_fit_ctx* c, int r0, int r1) {
     a.round_end = r1;
     a.deadline_ns = (c->bud.seconds > 0) ? c->t0_gpu + (unsigned long long)(c->bud.seconds * 1e9) : 0ull;
     const int clusters = plan_launch({c}, items, a);
-    if (a.ncl > 0 && c->xbar) CU(cudaMemsetAsync(c->xbar, 0, (size_t)c->pol.workers * 2 * 4, c->st));   // barriers, aborts
+    if (a.ncl > 0) CU(clear_group_state(c, c->st));
     CU(cudaEventRecord(c->ev_fork, c->st));
     CU(launch_worker(c->np, a, clusters, c->st));
     c->n_kernels++;
@@ -1115,7 +1123,7 @@ bm_status bm_fit_rounds_batch(bm_fit_ctx* const* fits, int32_t nfits, int32_t ro
             a.tpb = 256; a.k_smem = plan.k_smem;
             memcpy(a.cmap, plan.cmap, sizeof a.cmap);
             a.batch = (const WorkerArgs*)dargs;
-            if (c->xbar && cudaMemsetAsync(c->xbar, 0, (size_t)c->pol.workers * 2 * 4, st) != cudaSuccess)
+            if (clear_group_state(c, st) != cudaSuccess)
                 s = fail(BM_ECUDA, "barrier reset");
         }
         if (s) break;
@@ -1553,6 +1561,8 @@ static bm_status step_plan(bm_fit_ctx* c, const float* X, long long m, int n, in
     c->seed = seed;
     c->s_lo = c->s_hi = c->s_cap = std::max<long long>(s_cap, 1);
     c->w_lo = 0; c->w_hi = 1;
+    c->groups_ok = t_groups_ok;
+    c->rows_per_cta = g_rows_per_cta.load();
     c->max_cs = worker_max_cluster(c->np, k);
     c->cs = cluster_size(c->s_cap, c->max_cs, 0, rows_cap(c->np, k));
     if (c->cs == 0)
@@ -1626,6 +1636,15 @@ static bm_status stage_sample_and_centroids(bm_fit_ctx* c, const float* S_dev, l
     return BM_OK;
 }
 
+// A step call's launch: one worker, on as many clusters as a round would give
+// it (a group where the sample is large enough).
+static bm_status launch_step(bm_fit_ctx* c, WorkerArgs& a) {
+    const int clusters = plan_launch({c}, {{0, 0, a.step_s}}, a);
+    CU(clear_group_state(c, c->st));
+    CU(launch_worker(c->np, a, clusters, c->st));
+    return BM_OK;
+}
+
 bm_status bm_kmeanspp(const float* S_dev, int64_t s, int32_t n, float* C_inout_dev, int32_t k,
                       const uint8_t* degenerate_dev, int32_t trials, uint64_t seed, int32_t worker,
                       int32_t round, int32_t pass, void* stream) {
@@ -1640,7 +1659,7 @@ bm_status bm_kmeanspp(const float* S_dev, int64_t s, int32_t n, float* C_inout_d
     CU(cudaMemcpyAsync(c->deg, degenerate_dev, k, cudaMemcpyDeviceToDevice, c->st));
     WorkerArgs a = make_args(c, kModeStepKpp);
     a.trials = trials; a.step_s = s; a.step_worker = worker; a.step_round = round; a.step_pass = pass;
-    CU(launch_worker(c->np, a, 1, c->st));
+    if ((st = launch_step(c, a))) return st;
     CU(launch_unpad(c->Cw, k, n, c->np, C_inout_dev, c->st));
     Globals h;
     if ((st = read_globals(c, &h))) return st;
@@ -1661,10 +1680,9 @@ bm_status bm_lloyd(const float* S_dev, int64_t s, int32_t n, float* C_inout_dev,
     CU(cudaMemsetAsync(c->deg, 0, k, c->st));
     WorkerArgs a = make_args(c, kModeStepLloyd);
     a.max_lloyd = max_iter; a.tol = tol; a.step_s = s;
-    a.rows_cta = (int)((s + c->cs - 1) / c->cs);
     a.step_f = c->f_final; a.step_iters = (int*)c->L_buf;
     a.step_empty = empty_out_dev ? empty_out_dev : c->deg;
-    CU(launch_worker(c->np, a, 1, c->st));
+    if ((st = launch_step(c, a))) return st;
     CU(launch_unpad(c->Cw, k, n, c->np, C_inout_dev, c->st));
     double f = 0;
     int it = 0;

@@ -17,7 +17,7 @@ enum WorkerMode : int {
 // group): the clusters exchange their partial sums through global memory and
 // a barrier among the group's CTAs, which needs every CTA of the launch to be
 // resident at once (a cooperative launch).
-constexpr int kMaxGroup = 8;               // clusters per worker
+constexpr int kMaxGroup = 32;              // clusters per worker (a lane of a warp per cluster)
 constexpr int kMaxLaunchClusters = 160;    // entries of the cluster map
 
 struct WorkerArgs {
@@ -52,9 +52,9 @@ struct WorkerArgs {
     // are batch[f] (device memory, each with this launch's cs, rows_cta,
     // ncl and cmap); null: a launch for this fit alone
     const WorkerArgs* batch;
-    // group exchange in global memory (per worker; two parity halves)
-    long long* xpart;                 // W x 2 x kMaxGroup x k x NP x 3 words
-    int* xcnt;                        // W x 2 x kMaxGroup x k counts
+    // group exchange in global memory (per worker)
+    long long* xpart;                 // W x 3 x k x NP x 3 words: sums of the group, in turn (zero at launch)
+    int* xcnt;                        // W x 3 x k counts, likewise
     unsigned long long* xobj;         // W x 2 x kMaxGroup x 4 (objective partial, counters)
     unsigned* xbar;                   // W barrier counters (zero at launch)
     int* xabort;                      // W abort flags (zero at launch)

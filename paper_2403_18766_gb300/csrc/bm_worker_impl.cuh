@@ -87,6 +87,7 @@ struct Worker {
     int rank, cs, w, k, n;
     int gi, G, ctaW, nW;    // cluster gi of the worker's G clusters; CTA ctaW of its nW
     int xpar = 0;           // parity of the next group exchange
+    int xrot = 0;           // buffer of the next exchange of sums (0..2)
     int kpar = 0;           // parity of the next K-means++ exchange
     unsigned gepoch = 0;    // group barriers passed
     Grids g;
@@ -190,8 +191,13 @@ struct Worker {
         __threadfence();
     }
     __device__ bool group_aborted() const { return G > 1 && *(const volatile int*)(a.xabort + w) != 0; }
-    // Offsets of this worker's exchange slots (parity par, cluster q).
+    // Objective slot of cluster q (parity par).
     __device__ size_t xslot(int par, int q) const { return ((size_t)w * 2 + par) * kMaxGroup + q; }
+    // Sums of the group in buffer `rot`: words of (cluster j, dimension d), counts.
+    __device__ long long* xwords(int rot, int j, int d) const {
+        return a.xpart + ((((size_t)w * 3 + rot) * k + j) * NP + d) * kAccWords;
+    }
+    __device__ int* xcount(int rot, int j) const { return a.xcnt + ((size_t)w * 3 + rot) * k + j; }
 
     // cluster barrier that also orders global-memory writes
     __device__ void csync_global() {
@@ -651,14 +657,17 @@ struct Worker {
         }
     }
     __device__ double total_objective(unsigned __int128 F, unsigned long long I, unsigned long long R) {
-        if (G > 1) {
+        if (G > 1) {                                 // a lane per cluster
             F = 0; I = 0; R = 0;
-            for (int q = 0; q < G; ++q) {
-                const volatile unsigned long long* o = a.xobj + xslot(xpar, q) * 4;
-                F += ((unsigned __int128)o[1] << 64) | (unsigned __int128)o[0];
-                I += o[2];
-                R += o[3];
+            if ((int)(threadIdx.x & 31) < G) {
+                const volatile unsigned long long* o = a.xobj + xslot(xpar, threadIdx.x & 31) * 4;
+                F = ((unsigned __int128)o[1] << 64) | (unsigned __int128)o[0];
+                I = o[2];
+                R = o[3];
             }
+            F = warp_sum_u128(F);
+            I = warp_sum(I);
+            R = warp_sum(R);
         }
         if ((threadIdx.x & 31) == 0 && gi == 0) {
             if (I) atomicAdd(&a.glob->inexact, I);
@@ -666,18 +675,22 @@ struct Worker {
         }
         return u128_to_double(F, g.gf);
     }
-    // Owners publish their clusters' partial sums and counts (group only).
+    // Owners add their clusters' partial sums and counts to the group's (group
+    // only).  Three buffers take turns: one is added to before the barrier and
+    // read after it, and the one read after the barrier before is cleared
+    // then, two barriers before it is added to again.  (With a slot per
+    // cluster every owner read G slots one after the other.)
     __device__ void publish_sums() {
         if (G == 1) return;
         const int nOwned = (k - rank + cs - 1) / cs;
-        long long* dst = a.xpart + xslot(xpar, gi) * (size_t)k * NP * kAccWords;
-        int* dcnt = a.xcnt + xslot(xpar, gi) * (size_t)k;
         for (int e = threadIdx.x; e < nOwned * NP; e += TPB) {
             const int slot = e / NP, d = e % NP, j = rank + slot * cs;
             const long long* wd = sm.OACC + (size_t)e * kAccWords;
-            long long* o = dst + ((size_t)j * NP + d) * kAccWords;
-            o[0] = wd[0]; o[1] = wd[1]; o[2] = wd[2];
-            if (d == 0) dcnt[j] = sm.ocnt[slot];
+            unsigned long long* o = reinterpret_cast<unsigned long long*>(xwords(xrot, j, d));
+#pragma unroll
+            for (int i = 0; i < kAccWords; ++i)
+                if (wd[i]) atomicAdd(o + i, (unsigned long long)wd[i]);
+            if (d == 0 && sm.ocnt[slot]) atomicAdd(xcount(xrot, j), sm.ocnt[slot]);
         }
     }
     // Rank 0, one thread: the decision to every CTA of the cluster.
@@ -713,12 +726,16 @@ struct Worker {
                 const long long* wd = sm.OACC + (size_t)e * kAccWords;
                 V = (__int128)wd[0] + ((__int128)wd[1] << 32) + ((__int128)wd[2] << 64);
                 cntj = sm.ocnt[slot];
-            } else {                                 // the group's partials, in global memory
-                for (int q = 0; q < G; ++q) {
-                    const volatile long long* wd =
-                        a.xpart + (xslot(xpar, q) * (size_t)k * NP + (size_t)j * NP + d) * kAccWords;
-                    V += (__int128)wd[0] + ((__int128)wd[1] << 32) + ((__int128)wd[2] << 64);
-                    cntj += ((const volatile int*)a.xcnt)[xslot(xpar, q) * (size_t)k + j];
+            } else {                                 // the group's sums, in global memory
+                const long long* wd = xwords(xrot, j, d);
+                const long long w0 = __ldcg(wd), w1 = __ldcg(wd + 1), w2 = __ldcg(wd + 2);
+                cntj = __ldcg(xcount(xrot, j));
+                V = (__int128)w0 + ((__int128)w1 << 32) + ((__int128)w2 << 64);
+                if (gi == 0) {                       // the buffer of the exchange before: cleared for the next but one
+                    const int old = xrot == 0 ? 2 : xrot - 1;
+                    long long* z = xwords(old, j, d);
+                    z[0] = 0; z[1] = 0; z[2] = 0;
+                    if (d == 0) *xcount(old, j) = 0;
                 }
             }
             float c = sm.Ccur[(size_t)j * NP + d];
@@ -795,6 +812,7 @@ struct Worker {
                 }
             }
             xpar ^= 1;
+            xrot = xrot == 2 ? 0 : xrot + 1;
             trace_add(11, t_o);
             const long long t_b2 = clock64();
             cl.sync();                                       // updates + decision in every CTA
@@ -1194,11 +1212,11 @@ __global__ void __launch_bounds__(TPB, 512 / TPB) worker_kernel(const __grid_con
             W.prep_centroids();
             int iters = 0;
             const double f = W.lloyd(a.step_s, iters);
-            if (W.rank == 0 && threadIdx.x == 0) { *a.step_f = f; *a.step_iters = iters; }
-            if (W.rank == 0)
+            if (W.lead() && threadIdx.x == 0) { *a.step_f = f; *a.step_iters = iters; }
+            if (W.lead())
                 for (int j = threadIdx.x; j < W.k; j += TPB) a.step_empty[j] = W.sm.emptyall[j];
         }
-        if (W.rank == 0) W.store_centroids(a.Cw);
+        if (W.lead()) W.store_centroids(a.Cw);
         W.csync_global();
         return;
     }
@@ -1218,7 +1236,7 @@ __global__ void __launch_bounds__(TPB, 512 / TPB) worker_kernel(const __grid_con
         W.load_centroids(W.Cw_mine);
         W.prep_centroids();
         const double f = W.eval(s_opt);
-        if (W.rank == 0 && threadIdx.x == 0) a.f_final[w] = f;
+        if (W.lead() && threadIdx.x == 0) a.f_final[w] = f;
         W.cl.sync();
         return;
     }

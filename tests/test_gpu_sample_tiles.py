@@ -30,3 +30,24 @@ def test_lloyd_row_counts(n, k, s):
     ref = okm.lloyd(S, C0, 10, 1e-4)
     assert np.array_equal(C.cpu().numpy().view(np.uint32), ref["C"].view(np.uint32))
     assert f == ref["f"] and it == ref["iters"]
+
+
+@pytest.mark.parametrize("n,k,s", [(2, 5, 100_003), (16, 25, 70_001), (32, 50, 131_072), (64, 20, 40_000)])
+def test_step_calls_on_a_group_of_clusters(n, k, s):
+    """One worker on many clusters (the group's sums are added in three buffers in turn, so more than
+    three Lloyd exchanges) gives the bits of one cluster."""
+    S = torch.from_numpy(gaussian_mixture(s, n, k, seed=n + k)).cuda()
+    C0 = S[torch.linspace(0, s - 1, k).long().cuda()].clone()
+    outs = []
+    try:
+        for on in (1, 0):
+            native.set_worker_groups(on)
+            C, f, it, empty = native.lloyd(S, C0, 12, 0.0)
+            P = native.kmeanspp(S, C0, np.arange(k) % 2, 3, 5, 0, 0, 0)
+            outs.append((C, f, it, empty, P))
+    finally:
+        native.set_worker_groups(1)
+    a, b = outs
+    assert a[2] == b[2] >= 4 and a[1] == b[1] and torch.equal(a[3], b[3])
+    assert torch.equal(a[0].view(torch.int32), b[0].view(torch.int32))
+    assert torch.equal(a[4].view(torch.int32), b[4].view(torch.int32))
