@@ -215,6 +215,21 @@ __device__ __forceinline__ void acc_obj(unsigned __int128& acc, float d, int gf,
     }
 }
 
+// The common case of acc_obj: distances of at least lim = 2^(gf + 63) are whole
+// numbers of 2^(gf + 40), below 2^57 of them (a squared distance of data with
+// exponent Ex is below 2^(2 Ex + 11) = 2^(gf + 97)), so 64 of them add in 64
+// bits: three multiplications and a conversion instead of a 128-bit shift.
+struct FastSum {
+    float lim, s1, s2;                       // 2^-(gf + 40) as two exact factors
+    __device__ explicit FastSum(int gf) {
+        lim = ldexpf(1.f, max(gf + 63, -149));
+        const int e = -(gf + 40), e1 = min(max(e, -126), 127);
+        s1 = __int_as_float((unsigned)(e1 + 127) << 23);
+        s2 = ldexpf(1.f, e - e1);
+    }
+    __device__ __forceinline__ unsigned long long units(float d) const { return __float2ull_rz(d * s1 * s2); }
+};
+
 // A coordinate on the grid of the exact sums (unit 2^gx) as a signed 128-bit
 // integer.  Bits below the grid are truncated (counted in `inexact`); returns
 // false if |x| / 2^gx needs more than 96 bits (outside the grid's range; the

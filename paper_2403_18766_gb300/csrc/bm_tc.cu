@@ -329,15 +329,15 @@ tc_fullpass_kernel(const __nv_bfloat16* __restrict__ Xb, const float* __restrict
         const CertC cc = cert;
         const int b = warp >> 2, q4 = warp & 3;
         const unsigned trow = tmem + ((unsigned)(q4 * 32) << 16) + (unsigned)(b * sh.acc_stride);
+        const FastSum fs(gr.gf);
+        unsigned long long fast = 0;
+        int trips = 0;
         for (long long it = b;; it += NG) {
             const long long tile = blockIdx.x + it * grid;
             if (tile >= ntiles) break;
             const long long row = tile * kTcRows + q4 * 32 + lane;
             const float xx = row < m ? __ldg(xnorm + row) : 0.f;
-            int ok = 1;
-            if (lane == 0) ok = tc::wait(&accf[b], (unsigned)((it / NG) & 1), abort, g, sh.wait);
-            ok = __shfl_sync(0xffffffffu, ok, 0);
-            if (!ok) break;
+            if (!tc::wait_warp(&accf[b], (unsigned)((it / NG) & 1), abort, g, sh.wait)) break;
             tc::fence_after();
             // 1. the two least g (four chains); chunks of 16 columns,
             //    double-buffered
@@ -382,20 +382,24 @@ tc_fullpass_kernel(const __nv_bfloat16* __restrict__ Xb, const float* __restrict
             //    them, two words of bytes, the newest in the low byte)
             int j1 = 0, cnt = 0;
             unsigned lo = 0, hi = 0;
+            const float L = tc::next_up(lim);
             {
                 unsigned va[16], vb[16];
                 tc::ld16(trow, va);
                 for (int c0 = 0; c0 < k; c0 += 32) {
                     tc::wait_ld16(va);
                     if (c0 + 16 < k) tc::ld16(trow + (unsigned)(c0 + 16), vb);
-                    unsigned mk = (c0 + 16 <= k) ? tc::le_mask16<false>(va, ccb, c0, lim, 16)
-                                                 : tc::le_mask16<true>(va, ccb, c0, lim, k - c0);
+                    unsigned mk = (c0 + 16 <= k) ? tc::below_mask16<false>(0u, va, ccb, c0, L, 16)
+                                                 : tc::below_mask16<true>(0u, va, ccb, c0, L, k - c0);
                     if (c0 + 16 < k) {
                         tc::wait_ld16(vb);
                         if (c0 + 32 < k) tc::ld16(trow + (unsigned)(c0 + 32), va);
-                        mk |= ((c0 + 32 <= k) ? tc::le_mask16<false>(vb, ccb, c0 + 16, lim, 16)
-                                              : tc::le_mask16<true>(vb, ccb, c0 + 16, lim, k - c0 - 16)) << 16;
+                        mk = (c0 + 32 <= k) ? tc::below_mask16<false>(mk, vb, ccb, c0 + 16, L, 16)
+                                            : tc::below_mask16<true>(mk, vb, ccb, c0 + 16, L, k - c0 - 16);
+                    } else {
+                        mk <<= 16;
                     }
+                    mk = __brev(mk);                                  // bit i: column c0 + i
                     if (cnt == 0 && mk) j1 = c0 + __ffs(mk) - 1;      // a settled row's label
                     if (!close) cnt += mk != 0u;
                     unsigned mc = close ? mk : 0u;                    // a close call's candidates
@@ -425,11 +429,16 @@ tc_fullpass_kernel(const __nv_bfloat16* __restrict__ Xb, const float* __restrict
                         make_uint4((unsigned)row | all, (unsigned)cnt, lo, hi);
                 }
             }
-            if (row < m && !close) {
-                acc_obj(facc, fmaxf(0.f, xx + g1), gr.gf, inex);
-                if (labels) labels[row] = j1;
-            }
+            const bool settled = row < m && !close;
+            const float dv = fmaxf(0.f, xx + g1);
+            const bool quick = dv >= fs.lim && dv < __int_as_float(0x7f800000);
+            if (settled && quick) fast += fs.units(dv);
+            if (__any_sync(0xffffffffu, settled && !quick))
+                if (settled && !quick) acc_obj(facc, dv, gr.gf, inex);
+            if (settled && labels) labels[row] = j1;
+            if ((++trips & 63) == 0) { facc += (unsigned __int128)fast << 40; fast = 0; }
         }
+        facc += (unsigned __int128)fast << 40;
     }
 
     // teardown.  Without an abort every copy and every MMA was consumed by a

@@ -151,7 +151,7 @@ __device__ __forceinline__ void wait_ld() { asm volatile("tcgen05.wait::ld.sync.
 // ---------------------------------------------- epilogue helpers (g top-2)
 // Both tensor-core passes read, per row, g_j = fl(ccb_j - 2 acc_j) from the
 // accumulator columns in chunks of 16 and keep the two least g (pass 1),
-// then a bit mask of the columns with g <= lim (pass 2).
+// then a bit mask of the columns with g <= lim, i.e. below next_up(lim) (pass 2).
 
 // 16 tensor-memory columns in flight into r: the wait for them takes r as
 // operands, so that no use of r can be scheduled before the wait.
@@ -207,20 +207,33 @@ __device__ __forceinline__ void min2_chunk(float (&t1)[4], float (&t2)[4], const
         }
     }
 }
-// Pass 2 over the columns c0 .. c0 + 15 (the first `nv` when PART): bit i
-// set where g of column c0 + i is <= lim.
+// Pass 2 over the columns c0 .. c0 + 15 (the first `nv` when PART): mk moves
+// 16 bits up and takes, first column in the highest of them, whether g is
+// below L: the sign of g - L (exact in sign) by a funnel shift, which costs
+// one ALU operation per column instead of a compare and a predicated or
+// (10^7 x 64, k = 100, tau = 1e-3, the whole call with 64-bit distance sums and
+// waits by whole warps: 680 -> 643 us).
 template <bool PART>
-__device__ __forceinline__ unsigned le_mask16(const unsigned (&va)[16], const float* ccb, int c0, float lim, int nv) {
-    unsigned mk = 0;
+__device__ __forceinline__ unsigned below_mask16(unsigned mk, const unsigned (&va)[16], const float* ccb, int c0,
+                                                 float L, int nv) {
+    const float2 mL = make_float2(-L, -L);
 #pragma unroll
     for (int q = 0; q < 4; ++q) {
-        if (PART && 4 * q >= nv) break;
+        if (PART && 4 * q >= nv) { mk <<= 4; continue; }
         float e[4];
         g_quad(e, va, ccb, c0, q);
-#pragma unroll
-        for (int i = 0; i < 4; ++i) mk |= (e[i] <= lim) ? (1u << (4 * q + i)) : 0u;
+        const float2 d0 = __fadd2_rn(make_float2(e[0], e[1]), mL), d1 = __fadd2_rn(make_float2(e[2], e[3]), mL);
+        mk = __funnelshift_l(__float_as_uint(d0.x), mk, 1);
+        mk = __funnelshift_l(__float_as_uint(d0.y), mk, 1);
+        mk = __funnelshift_l(__float_as_uint(d1.x), mk, 1);
+        mk = __funnelshift_l(__float_as_uint(d1.y), mk, 1);
     }
-    return PART ? mk & ((1u << nv) - 1u) : mk;
+    return PART ? mk & ~((1u << (16 - nv)) - 1u) : mk;
+}
+// The float above v (v < next_up(w) exactly when v <= w); NaN for +inf and NaN.
+__device__ __forceinline__ float next_up(float v) {
+    const int b = __float_as_int(v);
+    return v == 0.f ? 0x1p-149f : __int_as_float(b < 0 ? b - 1 : b + 1);
 }
 
 // 32 lanes x 32 columns of 32-bit tensor-memory cells -> 32 registers per

@@ -263,12 +263,7 @@ tcx_fullpass_kernel(const __grid_constant__ CUtensorMap tmap, const float* __res
         unsigned char* xrow = xb + (size_t)b * kStage + r * 128;
         const unsigned trow = tmem + ((unsigned)(q4 * 32) << 16) + (unsigned)(b * sh.acc_stride);
         const int nw = MW == 1 ? 1 : sh.acc_stride >> 5;
-        // distances of at least 2^(gf + 63) add as one 64-bit integer in
-        // units of 2^(gf + 40) (exact; a distance is below 2^(gf + 97), so 64
-        // tiles fit); others, rare, go the general way
-        const float dlim = ldexpf(1.f, max(gr.gf + 63, -149));
-        const int eg = -(gr.gf + 40), e1 = min(max(eg, -126), 127);
-        const float s1 = __int_as_float((unsigned)(e1 + 127) << 23), s2 = ldexpf(1.f, eg - e1);
+        const FastSum fs(gr.gf);
         unsigned long long fast = 0;
         auto init_acc = [&]() {                              // the accumulator starts from ||c_j||^2
 #pragma unroll 1
@@ -411,8 +406,8 @@ tcx_fullpass_kernel(const __grid_constant__ CUtensorMap tmap, const float* __res
                     if (d < dv) { dv = d; lab = j; }
                 }
             }
-            const bool quick = dv >= dlim && dv < __int_as_float(0x7f800000);
-            if (valid && quick) fast += __float2ull_rz(dv * s1 * s2);
+            const bool quick = dv >= fs.lim && dv < __int_as_float(0x7f800000);
+            if (valid && quick) fast += fs.units(dv);
             if (__any_sync(0xffffffffu, valid && !quick))
                 if (valid && !quick) acc_obj(facc, dv, gr.gf, inex);
             if (valid && labels) labels[row] = lab;

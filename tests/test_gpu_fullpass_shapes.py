@@ -65,3 +65,16 @@ def test_rows_far_from_the_centroids_and_zero_rows():
 def test_choice_by_rows(m, n, k, tensor):
     X = gaussian_mixture_device(m, n, 6, seed=6)
     _same(X, X[:k].clone(), tensor)
+
+
+@pytest.mark.parametrize("k", [1, 5, 16, 17, 20, 31, 32, 33, 47, 49, 64, 97, 100, 129, 256])
+def test_precision_form_column_edges(k):
+    """The candidate masks of the BF16 pass at the edges of its chunks of 16 and 32 columns: the
+    certified form's labels are the exact pass's, and tau = inf gives its f too."""
+    X = gaussian_mixture_device(20_000, 50, max(1, k // 2), seed=k)
+    C = X[torch.linspace(0, 19_999, k).long().cuda()].clone()
+    P = native.PackedBF16(X)
+    Y, f, _ = native.assign(X, C)
+    assert torch.equal(native.assign_bf16(P, C, tau=0.0, certified=True)[0], Y)
+    Yi, fi, _ = native.assign_bf16(P, C, tau=float("inf"))
+    assert torch.equal(Yi, Y) and fi == f
