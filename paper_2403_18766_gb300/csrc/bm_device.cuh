@@ -404,6 +404,16 @@ __device__ __forceinline__ bool certified(float g1, float g2, float xn2, float x
     return gap > thr;                     // false for NaN; +inf gap (k = 1) passes
 }
 
+// A test without the square root that implies `certified`: 2 ||x|| cmax <=
+// ||x||^2 + cmax^2, with 2^-20 to spare for the roundings of both forms.  Rows
+// that fail it take the exact test, so the same rows are certified.
+__device__ __forceinline__ bool certified_quick(float g1, float g2, float xn2, const CertC& cc, float gB, float gp2) {
+    const float mag = __fmul_ru(__fadd_ru(xn2, __fmul_ru(2.f, cc.cmax2)), 1.f + 0x1p-20f);
+    const float B = __fmul_ru(gB, mag);
+    const float d1 = fmaxf(0.f, __fadd_ru(__fadd_ru(g1, B), xn2));
+    return __fsub_rd(g2, g1) > __fadd_ru(__fmul_ru(2.f, B), __fmul_ru(gp2, d1));
+}
+
 // ------------------------------------------------------------ block reduce
 template <typename T>
 __device__ __forceinline__ T warp_sum(T v) {

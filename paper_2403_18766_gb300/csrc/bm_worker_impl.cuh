@@ -287,10 +287,14 @@ struct Worker {
     // The CTA's rows of the first assignment of a Lloyd run, summed per
     // cluster without per-element atomics: the rows are bucketed by label
     // (counting sort of 16-bit row offsets in shared memory), each warp walks
-    // an equal share of the sorted rows with its lanes over (row, dimension),
-    // in batches whose loads are issued one batch ahead, keeps the exact sum
-    // in registers (two int64 parts of 48-bit-aligned pieces) and adds it to
-    // the owner's words once per cluster it meets.
+    // an equal share of the sorted rows one cluster at a time, its lanes over
+    // (row, dimension), in batches whose loads are issued one batch ahead,
+    // keeps the exact sum in registers and adds it to the owner's words once
+    // per cluster.  Bound by issue: about 60 instructions per step of 32
+    // values when every value was split in two 64-bit halves and every row's
+    // label compared.  A coordinate of at least 2^(gx + 71) (2^-24 of the
+    // largest |x|) is a whole number of 2^(gx + 48) and needs one half; the
+    // others take the second half for their batch.  @BUCKET@
     __device__ bool bucket_sums(long long lo, long long hi, unsigned int& inex) {
         const int nrows = (int)(hi - lo);
         __syncthreads();                                   // labs and lcnt complete
@@ -331,85 +335,105 @@ struct Worker {
         int dof[DPL];                                      // offsets of this lane's dimensions in a tile
 #pragma unroll
         for (int t = 0; t < DPL; ++t) dof[t] = (int)tile_at<NP>(0, d0 + t * LPR);
-        bool ok = true;
-        int cur = -1;                                      // cluster of this lane's running sum
-        long long shi[DPL], slo[DPL];
-#pragma unroll
-        for (int t = 0; t < DPL; ++t) shi[t] = slo[t] = 0;
-        // x 2^-gx as two exact power-of-two factors (each at most 2^127)
-        const int eg = -g.gx;
-        const int e1 = eg > 127 ? 127 : eg;
+        // x 2^-(gx + 48), below 2^48, as two exact power-of-two factors
+        const int eg = -(g.gx + 48);
+        const int e1 = min(max(eg, -126), 127);
         const float s1 = __int_as_float((unsigned)(e1 + 127) << 23);
-        const float s2 = __int_as_float((unsigned)(eg - e1 + 127) << 23);
-        // the rows of a batch (values and labels); the next batch is loaded
-        // while this one is converted and added
-        auto load_batch = [&](int q0, float (&xv)[U][DPL], int (&jl)[U]) {
+        const float s2 = ldexpf(1.f, eg - e1);
+        // a coordinate of at least 2^(gx + 71) is a whole number of 2^(gx + 48)
+        const float whole = ldexpf(1.f, max(g.gx + 71, -149));
+        float top = 0.f;                                   // largest |x| 2^-(gx + 48)
+        // the rows of a batch; the next batch is loaded while this one is
+        // converted and added
+        auto load_batch = [&](int q0, int q1, float (&xv)[U][DPL]) {
 #pragma unroll
             for (int u = 0; u < U; ++u) {
-                const int p = q0 + u * RPS;
-                const int r = p < b1 ? sm.rowlist[p] : 0;
-                jl[u] = p < b1 ? (int)sm.labs[r] : -1;
+                const int p = q0 + sub + u * RPS;
+                const int r = p < q1 ? sm.rowlist[p] : 0;
 #pragma unroll
-                for (int t = 0; t < DPL; ++t) {
-                    const int d = d0 + t * LPR;
-                    xv[u][t] = (p < b1 && d < n) ? S[tile_at<NP>(lo + r, 0) + dof[t]] : 0.f;
-                }
+                for (int t = 0; t < DPL; ++t)
+                    xv[u][t] = (p < q1 && d0 + t * LPR < n) ? S[tile_at<NP>(lo + r, 0) + dof[t]] : 0.f;
             }
         };
-        float xn[U][DPL];
-        int jn[U];
-        load_batch(b0 + sub, xn, jn);
-        for (int p0 = b0 + sub; p0 < b1; p0 += U * RPS) {
-            long long hv[U][DPL], lv[U][DPL];
-            int jv[U];
-            // the batch's coordinates on the grid, all at once, without
-            // branches: y = x 2^-gx exactly (|y| < 2^96 by the choice of gx),
-            // y = hf 2^48 + lf with hf an integer and lf the exact remainder,
-            // whose bits below the grid are truncated (and counted): the
-            // integer fixed_of gives, split at 2^48
-#pragma unroll
-            for (int u = 0; u < U; ++u) {
-                jv[u] = jn[u];
-#pragma unroll
-                for (int t = 0; t < DPL; ++t) {
-                    const float y = __fmul_rn(__fmul_rn(xn[u][t], s1), s2);
-                    const float hf = truncf(__fmul_rn(y, 0x1p-48f));
-                    const float lf = __fmaf_rn(-hf, 0x1p48f, y);
-                    const float lt = truncf(lf);
-                    inex += (lf != lt) ? 1u : 0u;
-                    ok &= fabsf(y) < 0x1p96f;
-                    hv[u][t] = __float2ll_rz(hf);
-                    lv[u][t] = __float2ll_rz(lt);
-                }
+        int j = 0;                                         // the cluster of sorted row b0
+        if (b0 < b1)
+            for (; j < k; j += 32) {
+                const unsigned past = __ballot_sync(0xffffffffu, sm.lstart[min(j + lane + 1, k)] > b0);
+                if (past) { j += __ffs(past) - 1; break; }
             }
-            if (p0 + U * RPS < b1) load_batch(p0 + U * RPS, xn, jn);
-            // rows are sorted by cluster: a running sum per lane, added to the
-            // owner's words when the cluster changes
+        int q0 = b0, q1 = b0 < b1 ? min(b1, sm.lstart[j + 1]) : b0;      // its rows in this warp's share
+        float xn[U][DPL];
+        if (q0 < q1) load_batch(q0, q1, xn);
+        while (q0 < q1) {                                  // one cluster at a time
+            long long shi[DPL], slo[DPL];
 #pragma unroll
-            for (int u = 0; u < U; ++u) {
-                if (jv[u] < 0) break;                      // past this warp's rows
-                if (jv[u] != cur) {
-                    if (cur >= 0)
+            for (int t = 0; t < DPL; ++t) shi[t] = slo[t] = 0;
+            const int jc = j;
+            int nq0 = q1, nq1 = q1;                        // the next cluster with rows here
+            if (q1 < b1) {
+                while (sm.lstart[++j + 1] <= q1) {}
+                nq1 = min(b1, sm.lstart[j + 1]);
+            }
+            bool low = false;                              // slo in use
+            for (int p0 = q0; p0 < q1; p0 += U * RPS) {
+                float xv[U][DPL];
+                bool part = false;
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+#pragma unroll
+                    for (int t = 0; t < DPL; ++t) {
+                        xv[u][t] = xn[u][t];
+                        part |= fabsf(xv[u][t]) < whole && xv[u][t] != 0.f;
+                    }
+                if (p0 + U * RPS < q1) load_batch(p0 + U * RPS, q1, xn);
+                else if (nq0 < nq1) load_batch(nq0, nq1, xn);
+                const bool any_part = __any_sync(0xffffffffu, part);
+                low |= any_part;
+#pragma unroll
+                for (int u = 0; u < U; ++u)
+#pragma unroll
+                    for (int t = 0; t < DPL; ++t) {
+                        const float y = __fmul_rn(__fmul_rn(xv[u][t], s1), s2);
+                        top = fmaxf(top, fabsf(y));
+                        shi[t] += __float2ll_rz(y);        // exact unless `part`: the rest below
+                    }
+                if (any_part) {
+                    // the parts below 2^(gx + 48), whose bits below the grid
+                    // are truncated (and counted): the integer fixed_of gives,
+                    // split at 2^48 (x 2^-gx in two factors of its own: the
+                    // remainder of a truncation at 2^48 is exact)
+                    const int f1 = min(-g.gx, 127);
+                    const float r1 = __int_as_float((unsigned)(f1 + 127) << 23);
+                    const float r2 = __int_as_float((unsigned)(-g.gx - f1 + 127) << 23);
+#pragma unroll
+                    for (int u = 0; u < U; ++u)
 #pragma unroll
                         for (int t = 0; t < DPL; ++t) {
-                            add_words(owner_words(cur, d0 + t * LPR),
-                                      ((__int128)shi[t] << 48) + (__int128)slo[t]);
-                            shi[t] = slo[t] = 0;
+                            const float y = __fmul_rn(__fmul_rn(xv[u][t], r1), r2);
+                            const float lf = __fmaf_rn(-truncf(__fmul_rn(y, 0x1p-48f)), 0x1p48f, y);
+                            const float lt = truncf(lf);
+                            inex += (lf != lt) ? 1u : 0u;
+                            slo[t] += __float2ll_rz(lt);
                         }
-                    cur = jv[u];
-                }
-#pragma unroll
-                for (int t = 0; t < DPL; ++t) {
-                    shi[t] += hv[u][t];
-                    slo[t] += lv[u][t];
                 }
             }
-        }
-        if (cur >= 0)
+            // the warp's sum of the cluster: over the rows of a step, then one
+            // lane per dimension adds it to the owner's words
 #pragma unroll
-            for (int t = 0; t < DPL; ++t)
-                add_words(owner_words(cur, d0 + t * LPR), ((__int128)shi[t] << 48) + (__int128)slo[t]);
-        return ok;
+            for (int o = LPR; o < 32; o <<= 1)
+#pragma unroll
+                for (int t = 0; t < DPL; ++t) {
+                    shi[t] += __shfl_xor_sync(0xffffffffu, shi[t], o);
+                    if (low) slo[t] += __shfl_xor_sync(0xffffffffu, slo[t], o);
+                }
+            if (sub == 0)
+#pragma unroll
+                for (int t = 0; t < DPL; ++t)
+                    add_words(owner_words(jc, d0 + t * LPR), ((__int128)shi[t] << 48) + (__int128)slo[t]);
+            q0 = nq0;
+            q1 = nq1;
+        }
+        return top < 0x1p48f;
     }
 
     // --------------------------------------------- a4/a5: assign + accumulate
@@ -421,16 +445,18 @@ struct Worker {
     // cluster to the new one.
     struct Tally {                       // what the rows of a thread add up to
         unsigned __int128 f = 0;
+        unsigned long long fast = 0;     // distances added in 64 bits (FastSum), at most 64 rows' worth
+        int rows = 0;
         unsigned int inex = 0, resc = 0;
         bool ok = true;
+        __device__ __forceinline__ void fold() { f += (unsigned __int128)fast << 40; fast = 0; rows = 0; }
     };
     // Rows row0 + 32 r + lane (r < R, below hi) of one warp; [nx0, nx1) are
     // the rows the warp takes next.
     template <int R>
     __device__ __forceinline__ void assign_rows(long long row0, long long lo, long long hi, long long nx0, long long nx1,
-                                                int mode, const CertC& cc, Tally& ty) {
+                                                int mode, const CertC& cc, const FastSum& fs, Tally& ty) {
         const float gB = a.gB, gp2 = a.gp2;
-        const int gf = g.gf;
         const int lane = threadIdx.x & 31;
         float2 m2x[R][NP / 2];                               // -2 x, dimension pairs
 #pragma unroll
@@ -496,11 +522,11 @@ struct Worker {
             const long long row = row0 + 32 * r + lane;
             const bool valid = row < hi;
             const float xn2 = xnorm2_up_m2x<NP>(m2x[r]);
-            const float xn = __fsqrt_ru(xn2);
             int lab = 0;
             float dv = 0.f;
             if (valid) {
-                if (certified(g1[r], g2[r], xn2, xn, cc, gB, gp2)) {
+                if (certified_quick(g1[r], g2[r], xn2, cc, gB, gp2) ||
+                    certified(g1[r], g2[r], xn2, __fsqrt_ru(xn2), cc, gB, gp2)) {
                     lab = j1[r];
                     dv = d32_m2x<NP>(m2x[r], sm.Ccur + (size_t)lab * NP);
                 } else {
@@ -511,7 +537,8 @@ struct Worker {
                         if (dj < dv) { dv = dj; lab = j; }
                     }
                 }
-                acc_obj(ty.f, dv, gf, ty.inex);
+                if (dv >= fs.lim && dv < __int_as_float(0x7f800000)) ty.fast += fs.units(dv);
+                else acc_obj(ty.f, dv, g.gf, ty.inex);
             }
             if (mode == 1) {
                 if (valid) {
@@ -562,13 +589,14 @@ struct Worker {
     // all warps instead of filling a few.
     template <int R>
     __device__ __forceinline__ bool assign_trip(int want, long long t0, long long t1, int nwant, long long lo,
-                                                long long hi, int mode, const CertC& cc, Tally& ty) {
+                                                long long hi, int mode, const CertC& cc, const FastSum& fs,
+                                                Tally& ty) {
         if constexpr (R > 1)
-            if (want < R) return assign_trip<R / 2>(want, t0, t1, nwant, lo, hi, mode, cc, ty);
+            if (want < R) return assign_trip<R / 2>(want, t0, t1, nwant, lo, hi, mode, cc, fs, ty);
         const int wid = threadIdx.x >> 5;
         const long long row0 = t0 + (long long)wid * 32 * R, nx0 = min(hi, t1 + (long long)wid * 32 * nwant);
         if (row0 < hi)
-            assign_rows<R>(row0, lo, hi, nx0, min(hi, nx0 + 32 * nwant), mode, cc, ty);
+            assign_rows<R>(row0, lo, hi, nx0, min(hi, nx0 + 32 * nwant), mode, cc, fs, ty);
         return true;
     }
     __device__ static int trip_rows(long long left) {        // R for the rows that are left
@@ -586,14 +614,18 @@ struct Worker {
         __syncthreads();
         const long long t_loop = clock64();
         const CertC cc = *sm.cert;
+        const FastSum fs(g.gf);
         Tally ty;
         const int lane = threadIdx.x & 31;
         for (long long t0 = lo; t0 < hi;) {                   // block-uniform
             const int R = trip_rows(hi - t0);
             const long long t1 = t0 + (long long)TPB * R;
-            assign_trip<RT>(R, t0, t1, trip_rows(hi - t1), lo, hi, mode, cc, ty);
+            if (ty.rows + R > 64) ty.fold();
+            ty.rows += R;
+            assign_trip<RT>(R, t0, t1, trip_rows(hi - t1), lo, hi, mode, cc, fs, ty);
             t0 = t1;
         }
+        ty.fold();
         unsigned __int128& facc = ty.f;
         unsigned int &inex = ty.inex, &resc = ty.resc;
         bool& ok = ty.ok;
