@@ -351,9 +351,11 @@ bm_status bm_assign(const float* X_dev, int64_t m, int32_t n, const float* C_dev
  * accumulation (tcgen05, kind::f16).  A row whose two least g differ by less
  * than tau * ||x||^2 is re-scored from the FP32 master X_dev with the exact
  * definition (FP32 direct form, lowest index on ties); otherwise its label is
- * the least g and its distance ||x||^2 + g (both in FP32).  f is the exact
- * sum of those distances rounded once to double; report->rescored_rows
- * counts re-scored rows.  A re-scored row is decided among its candidates,
+ * the least g and its distance ||x||^2 + g (both in FP32).  tau = infinity
+ * re-scores every row, also with one centroid (k = 1, where no second g
+ * exists and a finite tau re-scores none): labels and f are then those of
+ * bm_assign.  f is the exact sum of those distances rounded once to double;
+ * report->rescored_rows counts re-scored rows.  A re-scored row is decided among its candidates,
  * the centroids whose g lies within the certificate bound of
  * bm_assign_bf16_certified of the least g (they contain the exact-mode
  * argmin), or over all k when it has more than 8.  1 <= k <= 256.  Labels

@@ -187,8 +187,8 @@ bool tc_shape(int k, TcShape& s) {
 //     least in four interleaved chains, the rule, and for a close call a
 //     second read of the accumulator that lists its candidates; then the
 //     accumulator is handed back to the MMA issuer.
-// A close call (g2 - g1 < tau ||x||^2, or with `certify` a row whose BF16 gap
-// does not pass the certificate) goes to the queue with its candidates: the
+// A close call (g2 - g1 < tau ||x||^2, any row when tau is infinite, or with
+// `certify` a row whose BF16 gap does not pass the certificate) goes to the queue with its candidates: the
 // centroids whose g is at most fl_ru(g1 + thr), thr the certificate
 // threshold.  Any other centroid has a larger FP32 direct-form distance than
 // the centroid of g1 (the certificate's argument with the BF16 error factor),
@@ -330,6 +330,7 @@ tc_fullpass_kernel(const __nv_bfloat16* __restrict__ Xb, const float* __restrict
         const int b = warp >> 2, q4 = warp & 3;
         const unsigned trow = tmem + ((unsigned)(q4 * 32) << 16) + (unsigned)(b * sh.acc_stride);
         const FastSum fs(gr.gf);
+        const bool all_close = tau == __int_as_float(0x7f800000);   // also with one centroid, where g2 = +inf
         unsigned long long fast = 0;
         int trips = 0;
         for (long long it = b;; it += NG) {
@@ -368,7 +369,7 @@ tc_fullpass_kernel(const __nv_bfloat16* __restrict__ Xb, const float* __restrict
             }
             // 2. the rule; for a close call the certificate threshold (the
             //    bound on ||x||^2 is the BF16 norm x (1 + 2^-6))
-            bool close = row < m && !(g2 - g1 >= tau * xx);
+            bool close = row < m && (all_close || !(g2 - g1 >= tau * xx));
             float lim = g1;                 // the columns kept by pass 2: g <= lim
             if (row < m && (close || certify)) {
                 const float xn2 = __fmul_ru(xx, 1.0f + 0x1p-6f);
