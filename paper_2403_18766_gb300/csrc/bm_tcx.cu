@@ -35,6 +35,20 @@
 // is never accepted (subnormal data), and rows whose magnitudes come near the
 // FP32 range keep all columns.
 //
+// Shift.  That bound grows with the distance from the origin, the gaps between
+// distances do not: rows with a mean of a hundred standard deviations would
+// keep nearly all columns.  So the operands are x - u and c - u, u the mean of
+// up to 16 centroids, where that at least halves their mean ||c||^2 (any u
+// leaves ||x - c|| as it is); the direct form takes x and c as they are.
+// Each difference is rounded once, which changes ||c - u||^2 - 2 (x - u).(c - u)
+// by at most 2^-22 of the magnitudes in the bound (in tcx_gamma) and ||x - u||^2
+// by 2^-22 of itself (in xn2).  Up to 32 centroids (one mask word) keeping
+// every column costs less than the FP32-ALU pass, and nothing is shifted.
+// Measured, kernel alone, rows with a mean of 300 standard deviations: 10^6 x
+// 16, k = 200 2,110 -> 93 us; 2 10^6 x 32, k = 50 758 -> 99 us; 2 10^6 x 64, k =
+// 100 2,650 -> 207 us; centred rows, which pay for the test, 91 -> 93, 95 -> 97
+// and 189 -> 193 us.
+//
 // CTA roles (one CTA per SM, persistent over tiles blockIdx.x + i grid): the
 // warp after the epilogue warps issues the copies of X, the next one the
 // MMAs; NG epilogue warpgroups, group b taking the tiles i = b (mod NG) with
@@ -59,6 +73,7 @@
 #include <atomic>
 #include <cstdint>
 #include <mutex>
+#include <type_traits>
 
 #include <cuda.h>
 #include <cuda_bf16.h>
@@ -112,6 +127,7 @@ tcx_fullpass_kernel(const __grid_constant__ CUtensorMap tmap, const float* __res
                     Globals* g, float gB, float gp2, int incumbent, TxShape sh) {
     using K = TxK<NP>;
     constexpr int kStage = K::atoms * kTxAtomBytes;
+    constexpr bool kShift = MW > 1;              // see "Shift" in the file comment
     extern __shared__ __align__(1024) unsigned char smem_raw[];
     unsigned char* base = smem_raw + ((1024 - (tc::s_addr(smem_raw) & 1023)) & 1023);
     const int S = sh.stages;
@@ -127,7 +143,7 @@ tcx_fullpass_kernel(const __grid_constant__ CUtensorMap tmap, const float* __res
     __shared__ unsigned __int128 red128[kThreads / 32];
     __shared__ unsigned long long red64[kThreads / 32];
     __shared__ unsigned int redu[kThreads / 32];
-    __shared__ float cmax2_s;
+    __shared__ __align__(16) float mu_s[NP], sq_s[NP];               // the shift; mean squares
     __shared__ int wsel;
     __shared__ bool last;
 
@@ -148,12 +164,106 @@ tcx_fullpass_kernel(const __grid_constant__ CUtensorMap tmap, const float* __res
     if (warp == kMma) tc::tmem_alloc(&tmem_slot, (unsigned)sh.tmem_cols);
     __syncthreads();
     const float* C = Cw + (long long)wsel * k * cw;
-    // operands ch, cm of -2 c; the FP32 copy of -c; ||c||^2 and its bound
+    // copy of the CTA's it-th tile into stage s (the producer's lane 0)
+    auto copy_tile = [&](long long it, int s) {
+        const long long tile = blockIdx.x + it * gridDim.x;
+        if (sh.flat) {
+            const long long rows = min((long long)kTxRows, m - tile * kTxRows);
+            const unsigned bytes = (unsigned)(rows * n * 4) & ~15u;     // the rest by the row's thread
+            tc::expect_tx(&full[s], bytes);
+            if (bytes) tc::bulk_g2s(xs + (size_t)s * kStage, X + tile * kTxRows * n, bytes, &full[s]);
+        } else {
+            tc::expect_tx(&full[s], (unsigned)kStage);
+            for (int a = 0; a < K::atoms; ++a)
+                tc::tma_load_2d(xs + (size_t)s * kStage + (size_t)a * kTxAtomBytes, &tmap, 32 * a,
+                                (int)(tile * kTxRows), &full[s]);
+        }
+    };
+    long long issued = 0;             // producer: copies issued; MMA warp: tiles committed
+    if (warp == kProducer && lane == 0)                              // the first tiles are on their way meanwhile
+        for (; issued < S && blockIdx.x + issued * gridDim.x < (m + kTxRows - 1) / kTxRows; ++issued)
+            copy_tile(issued, (int)issued);
+    // the FP32 copy of -c and the shift
+    if (sh.cf)
+        for (int e = tid; e < k * NP; e += kThreads) {
+            const int j = e / NP, d = e % NP;
+            Cf[(size_t)j * K::CS + d] = d < cw ? -C[(size_t)j * cw + d] : 0.f;
+        }
+    if (kShift && tid < NP) {
+        const int cnt = min(k, 16);
+        const float w = 1.f / (float)cnt;
+        float mu = 0.f, sq = 0.f;
+#pragma unroll
+        for (int i = 0; i < 16; ++i)
+            if (i < cnt && tid < cw) {
+                const float c = C[(size_t)(i * k / cnt) * cw + tid];
+                mu = __fmaf_rn(c, w, mu);
+                sq = __fmaf_rn(c * w, c, sq);
+            }
+        mu_s[tid] = mu;
+        sq_s[tid] = sq;
+    }
+    // the operand buffers' columns that no row writes (NP = 8) are zero
+    if (NP < 16)
+        for (int e = tid; e < NG * kStage / 16; e += kThreads)
+            reinterpret_cast<uint4*>(xb)[e] = make_uint4(0u, 0u, 0u, 0u);
+    __syncthreads();
+    const float4* mu4 = reinterpret_cast<const float4*>(mu_s);
+    auto c4 = [&](int j, int q) {                                    // elements 4 q .. 4 q + 3 of centroid j
+        if (sh.cf) {
+            const float4 v = reinterpret_cast<const float4*>(Cf + (size_t)j * K::CS)[q];
+            return make_float4(-v.x, -v.y, -v.z, -v.w);
+        }
+        return 4 * q < cw ? __ldg(reinterpret_cast<const float4*>(C + (size_t)j * cw) + q)
+                          : make_float4(0.f, 0.f, 0.f, 0.f);
+    };
+    auto sub4 = [](const float4& v, const float4& u) {
+        return make_float4(__fsub_rn(v.x, u.x), __fsub_rn(v.y, u.y), __fsub_rn(v.z, u.z), __fsub_rn(v.w, u.w));
+    };
+    // Shift where that halves the mean ||c||^2 of those centroids, i.e. where
+    // ||u||^2 is more than half of it (every warp decides, alike).
+    bool shift = false;
+    if (kShift) {
+        float mu2 = 0.f, sq = 0.f;
+        for (int d = lane; d < NP; d += 32) {
+            mu2 = __fmaf_rn(mu_s[d], mu_s[d], mu2);
+            sq += sq_s[d];
+        }
+#pragma unroll
+        for (int o = 16; o > 0; o >>= 1) {
+            mu2 += __shfl_xor_sync(0xffffffffu, mu2, o);
+            sq += __shfl_xor_sync(0xffffffffu, sq, o);
+        }
+        shift = 2.f * mu2 > sq;
+    }
+    // ||c||^2 and its upper bound, a thread per centroid; the operands
+    static_assert(kThreads >= 256, "a thread per accumulator column");
+    {
+        float cc = 0.f, up = 0.f;
+        auto add = [&](float c) {
+            cc = __fmaf_rn(c, c, cc);
+            up = __fmaf_ru(c, c, up);
+        };
+        if (tid < k)
+#pragma unroll
+            for (int q = 0; q < NP / 4; ++q) {
+                float4 v = c4(tid, q);
+                if (shift) v = sub4(v, mu4[q]);
+                add(v.x); add(v.y); add(v.z); add(v.w);
+            }
+        if (tid < sh.acc_stride) CC[tid] = tid < k ? cc : __int_as_float(0x7f800000);
+        const unsigned mx = __reduce_max_sync(0xffffffffu, __float_as_uint(up));
+        if (lane == 0) redu[warp] = mx;
+    }
     for (int e = tid; e < sh.Npad * (K::KW / 8); e += kThreads) {
         const int j = e / (K::KW / 8), c = e % (K::KW / 8);
-        float v[8];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) v[i] = (j < k && 8 * c + i < cw) ? -2.f * C[(size_t)j * cw + 8 * c + i] : 0.f;
+        float v[8] = {};
+        if (j < k && 8 * c < NP) {
+            float4 a = c4(j, 2 * c), b = c4(j, 2 * c + 1);
+            if (shift) { a = sub4(a, mu4[2 * c]); b = sub4(b, mu4[2 * c + 1]); }
+            v[0] = -2.f * a.x; v[1] = -2.f * a.y; v[2] = -2.f * a.z; v[3] = -2.f * a.w;
+            v[4] = -2.f * b.x; v[5] = -2.f * b.y; v[6] = -2.f * b.z; v[7] = -2.f * b.w;
+        }
         uint4 h, l;
         tc::split_bf16(v, h, l);
         const int cm = K::atoms == 2 ? c : K::KW / 8 + c;            // chunk of cm in its row
@@ -161,67 +271,26 @@ tcx_fullpass_kernel(const __grid_constant__ CUtensorMap tmap, const float* __res
         *reinterpret_cast<uint4*>(cb + (K::atoms == 2 ? (size_t)sh.Npad * 128 : 0) + (size_t)j * 128 +
                                   ((cm ^ (j & 7)) << 4)) = l;
     }
-    if (sh.cf)
-        for (int e = tid; e < k * NP; e += kThreads) {
-            const int j = e / NP, d = e % NP;
-            Cf[(size_t)j * K::CS + d] = d < cw ? -C[(size_t)j * cw + d] : 0.f;
-        }
-    unsigned int mx = 0;
-    for (int j = tid; j < sh.acc_stride; j += kThreads) {
-        float acc = 0.f, up = 0.f;
-        if (j < k)
-            for (int d = 0; d < cw; ++d) {
-                const float c = C[(size_t)j * cw + d];
-                acc = __fmaf_rn(c, c, acc);
-                up = __fmaf_ru(c, c, up);
-            }
-        CC[j] = (j < k) ? acc : __int_as_float(0x7f800000);
-        mx = max(mx, __float_as_uint(up));
-    }
-    mx = __reduce_max_sync(0xffffffffu, mx);
-    if (lane == 0) redu[warp] = mx;
-    // the operand buffers' columns that no row writes (NP = 8) are zero
-    if (NP < 16)
-        for (int e = tid; e < NG * kStage / 16; e += kThreads)
-            reinterpret_cast<uint4*>(xb)[e] = make_uint4(0u, 0u, 0u, 0u);
     tc::fence_proxy_async();
     tc::fence_before();
     __syncthreads();
     tc::fence_after();
-    if (tid == 0) {
-        unsigned int mm = 0;
-        for (int i = 0; i < kThreads / 32; ++i) mm = max(mm, redu[i]);
-        cmax2_s = __uint_as_float(mm);
-    }
-    __syncthreads();
     const unsigned tmem = tmem_slot;
     const long long ntiles = (m + kTxRows - 1) / kTxRows;
     const long long grid = gridDim.x;
 
     unsigned __int128 facc = 0;
     unsigned int inex = 0, resc = 0;
-    long long issued = 0;             // producer: copies issued; MMA warp: tiles committed
     if (warp == kProducer) {
         // ---------------------------------------------------------- producer
         if (lane == 0) {
-            long long it = 0;
-            int s = 0;
-            unsigned ph = 0;                                // (it / S) & 1, kept incrementally
+            long long it = issued;
+            int s = (int)(it % S);
+            unsigned ph = (unsigned)(it / S) & 1u;          // (it / S) & 1, kept incrementally
             for (;; ++it) {
-                const long long tile = blockIdx.x + it * grid;
-                if (tile >= ntiles) break;
+                if (blockIdx.x + it * grid >= ntiles) break;
                 if (it >= S && !tc::wait(&empty[s], ph ^ 1u, abort, g, sh.wait)) break;
-                if (sh.flat) {
-                    const long long rows = min((long long)kTxRows, m - tile * kTxRows);
-                    const unsigned bytes = (unsigned)(rows * n * 4) & ~15u;     // the rest by the row's thread
-                    tc::expect_tx(&full[s], bytes);
-                    if (bytes) tc::bulk_g2s(xs + (size_t)s * kStage, X + tile * kTxRows * n, bytes, &full[s]);
-                } else {
-                    tc::expect_tx(&full[s], (unsigned)kStage);
-                    for (int a = 0; a < K::atoms; ++a)
-                        tc::tma_load_2d(xs + (size_t)s * kStage + (size_t)a * kTxAtomBytes, &tmap, 32 * a,
-                                        (int)(tile * kTxRows), &full[s]);
-                }
+                copy_tile(it, s);
                 if (++s == S) { s = 0; ph ^= 1u; }
             }
             issued = it;
@@ -256,8 +325,11 @@ tcx_fullpass_kernel(const __grid_constant__ CUtensorMap tmap, const float* __res
         }
     } else {
         // --------------------------------------------------- epilogue groups
+        // (a body of its own for shifted rows: a branch per row cost the
+        // unshifted ones 2 to 5%)
+        auto epilogue = [&](auto shifted) __attribute__((always_inline)) {
         const Grids gr = grids_from_maxbits(g->maxbits);
-        const float cmax2 = cmax2_s;
+        const float cmax2 = __uint_as_float(__reduce_max_sync(0xffffffffu, lane < kThreads / 32 ? redu[lane] : 0u));
         const int b = warp >> 2, q4 = warp & 3;
         const int r = q4 * 32 + lane;                        // row within the tile = TMEM lane
         unsigned char* xrow = xb + (size_t)b * kStage + r * 128;
@@ -311,6 +383,13 @@ tcx_fullpass_kernel(const __grid_constant__ CUtensorMap tmap, const float* __res
                 float v[8];
 #pragma unroll
                 for (int i = 0; i < 8; ++i) v[i] = x[8 * c + i];
+                if constexpr (decltype(shifted)::value) {
+                    const float4 u0 = mu4[2 * c], u1 = mu4[2 * c + 1];
+                    v[0] = __fsub_rn(v[0], u0.x); v[1] = __fsub_rn(v[1], u0.y);
+                    v[2] = __fsub_rn(v[2], u0.z); v[3] = __fsub_rn(v[3], u0.w);
+                    v[4] = __fsub_rn(v[4], u1.x); v[5] = __fsub_rn(v[5], u1.y);
+                    v[6] = __fsub_rn(v[6], u1.z); v[7] = __fsub_rn(v[7], u1.w);
+                }
 #pragma unroll
                 for (int i = 0; i < 8; i += 2)
                     n2 = __ffma2_ru(make_float2(v[i], v[i + 1]), make_float2(v[i], v[i + 1]), n2);
@@ -326,7 +405,8 @@ tcx_fullpass_kernel(const __grid_constant__ CUtensorMap tmap, const float* __res
             if (lane == 0) tc::arrive(&conv[b]);
             s += NG;
             while (s >= S) { s -= S; ++use; }
-            const float xn2 = __fadd_ru(n2.x, n2.y);
+            float xn2 = __fadd_ru(n2.x, n2.y);
+            if constexpr (decltype(shifted)::value) xn2 = __fmul_ru(xn2, 1.f + 0x1p-21f);
             const float mag = __fadd_ru(xn2, __fmul_ru(2.f, cmax2));      // >= cmax^2 + 2 ||x|| cmax
             const float B = __fmul_ru(gB, mag);
             // 2. the accumulator: least g, then the columns within the threshold
@@ -414,6 +494,9 @@ tcx_fullpass_kernel(const __grid_constant__ CUtensorMap tmap, const float* __res
             if ((u & 63) == 63) { facc += (unsigned __int128)fast << 40; fast = 0; }
         }
         facc += (unsigned __int128)fast << 40;
+        };
+        if (kShift && shift) epilogue(std::true_type{});
+        else epilogue(std::false_type{});
     }
 
     // teardown.  Without an abort every copy and every MMA was consumed by a
@@ -537,7 +620,8 @@ cudaError_t launch_t(const CUtensorMap& tm, const float* X, long long m, int n, 
 
 // Certificate factor of the split products (see the file comment).
 float tcx_gamma(int steps) {
-    return 1.25f * (3.0f * 0x1p-16f * (1.f + 0x1p-6f) + (3 * steps) * 17 * 0x1p-23f * (1.f + 0x1p-6f) + 0x1p-18f);
+    return 1.25f * (3.0f * 0x1p-16f * (1.f + 0x1p-6f) + (3 * steps) * 17 * 0x1p-23f * (1.f + 0x1p-6f) + 0x1p-18f +
+                    0x1p-21f);
 }
 
 // Limits of the bounded waits of the next launches (process-wide).
