@@ -450,10 +450,14 @@ int32_t bm_last_fullpass_impl(void);
  *   clusters the device can hold beyond one per worker go to the workers
  *   with the most sample rows per CTA, so a large sample spans up to 32
  *   clusters (256 CTAs) that add up their exact partial sums in global memory
- *   with a barrier among the group's CTAs (bm_kmeanspp and bm_lloyd: the one
- *   worker has the device to itself); rows per CTA then stay about
+ *   with a barrier among the group's CTAs; rows per CTA then stay about
  *   equal across workers.  Each such barrier is bounded (a few seconds):
  *   when one runs out the round returns BM_ETIMEOUT.
+ *   bm_kmeanspp and bm_lloyd: the one worker takes as many clusters as its
+ *   rows fill, up to the device divided by the bm_kmeanspp and bm_lloyd calls
+ *   in progress on it, so calls from several threads on their own streams run
+ *   side by side.  A launch starts once all of its CTAs fit beside what else
+ *   runs on the device; with bm_set_worker_groups(0) it needs one cluster.
  *   Otherwise (bm_set_worker_groups(0), more workers than resident clusters,
  *   or bm_set_big_clusters(1)): one cluster per worker, all of the size the
  *   largest sample needs (the cluster tile below), in the same launch.
