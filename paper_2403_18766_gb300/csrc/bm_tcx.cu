@@ -10,7 +10,8 @@
 //     likewise into ch and cm; a tile of 128 rows takes the MMAs xh.ch, xh.cm
 //     and xm.ch (tcgen05.mma kind::f16, BF16 operands, M = 128, N = k rounded
 //     up to 16, K = 16) on top of an FP32 accumulator in tensor memory that
-//     starts from ||c_j||^2, so the accumulator is g_j = ||c_j||^2 - 2 x.c_j;
+//     starts from ||c_j||^2 (a little less, see below), so the accumulator is
+//     g_j = ||c_j||^2 - 2 x.c_j;
 //   * the epilogue takes the least g of a row from the tensor-memory load
 //     itself (tcgen05.ld.red, sm_103a), adds the certificate's threshold and
 //     keeps the bit mask of the columns below: no other centroid can be the
@@ -28,14 +29,30 @@
 // accumulation is taken to add at most (K + 1) 2^-23 of the magnitude
 // accumulated so far per MMA instruction (products aligned and truncated once
 // against the largest term, then added): 3 ksteps instructions on magnitudes
-// of at most (1 + 2^-6)(cmax^2 + 2 ||x|| cmax).  ||c_j||^2 itself is an FP32
-// FMA chain (64 2^-24).  tcx_gamma sums these with a quarter to spare; it
-// bounds |g_j - (||c_j||^2 - 2 x.c_j)| by gB (cmax^2 + 2 ||x|| cmax), and
-// 2 ||x|| cmax <= ||x||^2 + cmax^2 spares the square root.  A gap below 2^-60
-// is never accepted (subnormal data), and rows whose magnitudes come near the
-// FP32 range keep all columns.
+// of at most (1 + 2^-6)(||c_j||^2 + 2 ||x|| ||c_j||).  ||c_j||^2 itself is an
+// FP32 FMA chain (64 2^-24).  tcx_gamma sums these with a quarter to spare; it
+// bounds |g_j - (||c_j||^2 - 2 x.c_j)| by gB (||c_j||^2 + 2 ||x|| ||c_j||), at
+// most gB (2 ||c_j||^2 + ||x||^2).
 //
-// Shift.  That bound grows with the distance from the origin, the gaps between
+// Threshold.  With the largest ||c||^2 in that bound, one far centroid would
+// make every row keep the centroids near it.  So the accumulator starts from
+// (1 - 2 gB) ||c_j||^2 (a hair less): then the squared distance D_j =
+// ||x||^2 + ||c_j||^2 - 2 x.c_j is at least ||x||^2 + g_j - gB ||x||^2, and for
+// the centroid of the least g, g1, at most
+//   D <= ||x||^2 + g1 + gB (||x||^2 + 4.1 N),   N = ||c||^2 of that centroid.
+// N <= (||x|| + sqrt D)^2 <= 1.5 ||x||^2 + 3 D, hence (gB < 2^-12)
+//   D <= d1 = 1.006 (max(0, ||x||^2 + g1) + 7.2 gB ||x||^2),
+// and a centroid whose g exceeds g1 by more than
+//   thr = gB (2 ||x||^2 + 4.1 min(max ||c||^2, 1.5 ||x||^2 + 3 d1)) + gp2 d1
+// has a D larger by gp2 D and more, so a larger direct form (its relative
+// error is in gp2).  A gap below 2^-60 is never accepted (subnormal data), and
+// rows whose magnitudes come near the FP32 range keep all columns.  Up to 32
+// centroids the minimum is left out (a mask of one word costs little).
+// Measured (the call, log-normal rows with sigma = 3, k = 200) with the largest
+// ||c||^2 alone in the bound and so: 10^6 x 16 1,886 and 153 us, 10^6 x 32 1,899
+// and 191 us, 5 10^6 x 8 8,802 and 514 us.
+//
+// Shift.  The bound grows with the distance from the origin, the gaps between
 // distances do not: rows with a mean of a hundred standard deviations would
 // keep nearly all columns.  So the operands are x - u and c - u, u the mean of
 // up to 16 centroids, where that at least halves their mean ||c||^2 (any u
@@ -135,7 +152,7 @@ tcx_fullpass_kernel(const __grid_constant__ CUtensorMap tmap, const float* __res
     unsigned char* xb = xs + (size_t)S * kStage;                     // xh | xm, one per group
     unsigned char* cb = xb + (size_t)NG * kStage;                    // ch | cm
     float* Cf = reinterpret_cast<float*>(cb + (size_t)K::atoms * sh.Npad * 128);   // -C (sh.cf)
-    float* CC = Cf + (sh.cf ? (size_t)k * K::CS : 0);                // ||c_j||^2, +inf past k
+    float* CC = Cf + (sh.cf ? (size_t)k * K::CS : 0);                // (1 - 2 gB) ||c_j||^2, +inf past k
     constexpr int kEpi = 4 * NG, kProducer = kEpi, kMma = kEpi + 1, kThreads = tx_threads(NG);
     __shared__ __align__(8) unsigned long long full[kTxMaxStages], empty[kTxMaxStages], conv[NG], accf[NG];
     __shared__ unsigned tmem_slot;
@@ -251,7 +268,7 @@ tcx_fullpass_kernel(const __grid_constant__ CUtensorMap tmap, const float* __res
                 if (shift) v = sub4(v, mu4[q]);
                 add(v.x); add(v.y); add(v.z); add(v.w);
             }
-        if (tid < sh.acc_stride) CC[tid] = tid < k ? cc : __int_as_float(0x7f800000);
+        if (tid < sh.acc_stride) CC[tid] = tid < k ? cc * (1.f - 2.02f * gB) : __int_as_float(0x7f800000);
         const unsigned mx = __reduce_max_sync(0xffffffffu, __float_as_uint(up));
         if (lane == 0) redu[warp] = mx;
     }
@@ -330,6 +347,9 @@ tcx_fullpass_kernel(const __grid_constant__ CUtensorMap tmap, const float* __res
         auto epilogue = [&](auto shifted) __attribute__((always_inline)) {
         const Grids gr = grids_from_maxbits(g->maxbits);
         const float cmax2 = __uint_as_float(__reduce_max_sync(0xffffffffu, lane < kThreads / 32 ? redu[lane] : 0u));
+        // (each constant of the threshold has 2^-9 of itself to spare for roundings)
+        const float k_max = fmaxf(4.11f * gB * cmax2, 0x1p-60f);
+        const float k_gp = gp2 * (1.f + 0x1p-9f), k_own = 12.4f * gB + k_gp;
         const int b = warp >> 2, q4 = warp & 3;
         const int r = q4 * 32 + lane;                        // row within the tile = TMEM lane
         unsigned char* xrow = xb + (size_t)b * kStage + r * 128;
@@ -337,7 +357,7 @@ tcx_fullpass_kernel(const __grid_constant__ CUtensorMap tmap, const float* __res
         const int nw = MW == 1 ? 1 : sh.acc_stride >> 5;
         const FastSum fs(gr.gf);
         unsigned long long fast = 0;
-        auto init_acc = [&]() {                              // the accumulator starts from ||c_j||^2
+        auto init_acc = [&]() {                              // the accumulator starts from CC
 #pragma unroll 1
             for (int w = 0; w < nw; ++w) tc::st32_shared(trow + 32u * w, CC + 32 * w);
             tc::wait_st();
@@ -407,8 +427,11 @@ tcx_fullpass_kernel(const __grid_constant__ CUtensorMap tmap, const float* __res
             while (s >= S) { s -= S; ++use; }
             float xn2 = __fadd_ru(n2.x, n2.y);
             if constexpr (decltype(shifted)::value) xn2 = __fmul_ru(xn2, 1.f + 0x1p-21f);
-            const float mag = __fadd_ru(xn2, __fmul_ru(2.f, cmax2));      // >= cmax^2 + 2 ||x|| cmax
-            const float B = __fmul_ru(gB, mag);
+            // what the threshold takes from ||x||^2
+            const float d_lo = __fmul_ru(7.3f * gB, xn2);
+            const float t_max = __fmaf_ru(2.01f * gB, xn2, k_max);
+            const bool sane = t_max < 0x1p106f;               // ||x||^2 + 2 cmax^2 below 2^122; else: every column
+            const float t_own = fmaxf(__fmul_ru(8.2f * gB, xn2), 0x1p-60f);
             // 2. the accumulator: least g, then the columns within the threshold
             if (!tc::wait_warp(&accf[b], (unsigned)(u & 1), abort, g, sh.wait)) break;
             tc::fence_after();
@@ -421,11 +444,10 @@ tcx_fullpass_kernel(const __grid_constant__ CUtensorMap tmap, const float* __res
                 g1 = fminf(g1, mn);
             }
             // every column with g <= g1 + thr lies strictly below L
-            const float d1 = fmaxf(0.f, __fadd_ru(__fadd_ru(g1, B), xn2));
-            const float thr = __fmul_ru(fmaxf(__fadd_ru(__fmul_ru(2.f, B), __fmul_ru(gp2, d1)), 0x1p-60f),
-                                        1.f + 0x1p-20f);
+            const float d1 = __fmaf_ru(1.007f, fmaxf(0.f, __fadd_ru(g1, xn2)), d_lo);
+            float thr = __fmaf_ru(k_gp, d1, t_max);
+            if (MW > 1) thr = fminf(thr, __fmaf_ru(k_own, d1, t_own));
             const float L = __fadd_ru(g1, thr);
-            const bool sane = mag < 0x1p120f;                 // else: every column
             int cnt = 0;
 #pragma unroll
             for (int w = 0; w < MW; ++w) {
