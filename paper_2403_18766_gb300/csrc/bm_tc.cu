@@ -48,13 +48,17 @@ constexpr int kTcK = 64;               // packed row width (BF16 elements)
 // from there (so the norm's chain stays in a thread, and reads and writes of
 // shared memory meet no bank conflicts: the swizzle spreads the chunks), and
 // the packed tile, 16 KB in one piece of Xb, is written with coalesced 16-byte
-// stores.  6 CTAs per SM overlap one another's phases.
+// stores.  4 CTAs per SM (registers) overlap one another's phases; chunks past
+// n are not read.
 // Measured on 10^7 x 64 (3.88 GB moved): 2,677 us when every thread read its
 // own pieces of rows and the norms came from a second walk, now 589 us (6.6
-// TB/s).
+// TB/s).  Rows that are no multiple of 16 bytes come by 4-byte loads, 16 of a
+// thread in flight.  Pack calls on 4 10^6 rows, with one such load in flight, 3
+// CTAs per SM and all 64 columns zeroed and read of every row, against this:
+// n = 31 540 -> 249 us, 63 876 -> 368, 16 230 -> 187, 4 209 -> 157, 64 297 -> 274.
 constexpr int kPkRows = 128;
 constexpr int kPkStride = kTcK + 4;
-__global__ void __launch_bounds__(kPkRows) pack_bf16_kernel(const float* __restrict__ X, long long m, int n,
+__global__ void __launch_bounds__(kPkRows, 4) pack_bf16_kernel(const float* __restrict__ X, long long m, int n,
                                                             long long m_pad, __nv_bfloat16* __restrict__ Xb,
                                                             float* __restrict__ norms) {
     __shared__ __align__(16) float xs[kPkRows * kPkStride];
@@ -64,7 +68,6 @@ __global__ void __launch_bounds__(kPkRows) pack_bf16_kernel(const float* __restr
     // e / per for e < 2^13 by multiplication: (2^20 / per rounded up) e 2^-20
     const unsigned inv = ((1u << 20) + per - 1) / per;
     unsigned int mx = 0;
-    for (int i = tid; i < kPkRows * kPkStride; i += kPkRows) xs[i] = 0.f;      // columns n .. 63
     for (long long tile = blockIdx.x; tile < m_pad / kPkRows; tile += gridDim.x) {
         const long long r0 = tile * kPkRows;
         const int rows = (int)min((long long)kPkRows, m - r0);
@@ -88,9 +91,22 @@ __global__ void __launch_bounds__(kPkRows) pack_bf16_kernel(const float* __restr
                 }
             }
         } else {
-            for (int e = tid; e < kPkRows * per; e += kPkRows) {
-                const int r = (int)((unsigned)e * inv >> 20);
-                xs[r * kPkStride + e - r * per] = e < rows * per ? __ldg(src + e) : 0.f;
+            constexpr int U = 16;                         // loads in flight
+            for (int e0 = tid; e0 < kPkRows * per; e0 += U * kPkRows) {
+                float w[U];
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const int e = e0 + u * kPkRows;
+                    w[u] = e < rows * per ? __ldg(src + e) : 0.f;
+                }
+#pragma unroll
+                for (int u = 0; u < U; ++u) {
+                    const int e = e0 + u * kPkRows;
+                    if (e < kPkRows * per) {
+                        const int r = (int)((unsigned)e * inv >> 20);
+                        xs[r * kPkStride + e - r * per] = w[u];
+                    }
+                }
             }
         }
         __syncthreads();
@@ -100,9 +116,16 @@ __global__ void __launch_bounds__(kPkRows) pack_bf16_kernel(const float* __restr
         float acc = 0.f;
 #pragma unroll
         for (int c = 0; c < kTcK / 8; ++c) {
+            if (8 * c >= n) {
+                pk[c] = make_uint4(0u, 0u, 0u, 0u);
+                continue;
+            }
             const float4 a = *reinterpret_cast<const float4*>(xs + tid * kPkStride + 8 * c);
             const float4 b = *reinterpret_cast<const float4*>(xs + tid * kPkStride + 8 * c + 4);
-            const float x[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+            float x[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+            if (8 * c + 8 > n)                            // columns n .. are not in the tile
+#pragma unroll
+                for (int i = 1; i < 8; ++i) x[i] = 8 * c + i < n ? x[i] : 0.f;
             __align__(16) __nv_bfloat16 v[8];
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
@@ -123,11 +146,6 @@ __global__ void __launch_bounds__(kPkRows) pack_bf16_kernel(const float* __restr
             uint4* dst = reinterpret_cast<uint4*>(Xb + r0 * kTcK);
 #pragma unroll
             for (int u = 0; u < kTcK / 8; ++u) dst[tid + u * kPkRows] = ps[tid + u * kPkRows];
-            if (n < kTcK) {                               // the staged chunks covered the zero columns
-                __syncthreads();
-                for (int i = tid; i < kPkRows * kTcK / 4; i += kPkRows)
-                    reinterpret_cast<float4*>(xs)[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-            }
         }
     }
     // norms[m_pad] = max |x| (bits; non-finite values compare above all finite ones)

@@ -73,3 +73,23 @@ def test_scan_of_an_unaligned_sample(s, shift):
     b = native.lloyd(torch.from_numpy(x).cuda(), C, max_iter=3)
     assert torch.equal(a[0], b[0]) and a[1] == b[1] and a[2] == b[2]
     assert np.isfinite(a[1])
+
+
+@pytest.mark.parametrize("n", [31, 61])
+def test_pack_of_odd_widths_keeps_up_with_even_ones(n):
+    """Rows that are no multiple of 16 bytes take at most half as long again as those one wider."""
+    def us(X):
+        for _ in range(3):
+            native.PackedBF16(X)
+        best = 1e9
+        for _ in range(8):
+            a, b = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+            a.record()
+            native.PackedBF16(X)
+            b.record()
+            b.synchronize()
+            best = min(best, a.elapsed_time(b) * 1e3)
+        return best
+
+    m = 4_000_000
+    assert us(torch.randn((m, n), device="cuda")) <= 1.5 * us(torch.randn((m, n + 1), device="cuda"))
