@@ -763,7 +763,7 @@ bm_status round_samples(bm_fit_ctx* c, int r0) {
         sa.rnd = r0;
         CU(launch_sample(c->np, sa, (c->w_hi - c->w_lo) * (c->pol.passes + 1), c->st));
         span_end(c, sp_s);
-        c->n_kernels++;
+        c->n_kernels += sample_kernels(sa);
     }
     c->prefetched = -1;
     return BM_OK;
@@ -783,7 +783,7 @@ bm_status round_prefetch(bm_fit_ctx* c, int r0) {
         CU(launch_sample(c->np, sa, (c->w_hi - c->w_lo) * (c->pol.passes + 1), c->sst));
         span_end(c, sp_s);
         CU(cudaEventRecord(c->ev_sdone, c->sst));
-        c->n_kernels++;
+        c->n_kernels += sample_kernels(sa);
         c->prefetched = r0 + 1;
     }
     return BM_OK;
@@ -1196,7 +1196,7 @@ bm_status bm_fit_recheck(bm_fit_ctx* c, int64_t s_opt, double* f_out_host) {
     WorkerArgs a = make_args(c, kModeFinalEval);
     a.worker_base = c->w_lo;
     CU(launch_worker(c->np, a, c->w_hi - c->w_lo, c->st));
-    c->n_kernels += 2;
+    c->n_kernels += sample_kernels(sa) + 1;
     span_end(c, sp);
     CU(cudaMemcpyAsync(f_out_host, c->f_final + c->w_lo, (size_t)(c->w_hi - c->w_lo) * 8, cudaMemcpyDeviceToHost,
                        c->st));
@@ -1240,7 +1240,7 @@ static bm_status fit_finish(bm_fit_ctx* c, float* C_out_dev, int32_t* labels_out
     if ((s = make_sample_args(c, kSampleFinal, 1, 0, false, c->st, sa))) return s;
     CU(launch_sample(c->np, sa, 1, c->st));
     CU(launch_worker(c->np, a, c->pol.workers, c->st));
-    c->n_kernels += 2;
+    c->n_kernels += sample_kernels(sa) + 1;
     span_end(c, sp);
     if (full_pass && (s = run_fullpass(c, c->f_final, labels_out_dev, 1))) return s;
     CU(launch_select_unpad(c->Cw, c->f_final, c->pol.workers, c->k, c->n, c->np, C_out_dev, c->st));

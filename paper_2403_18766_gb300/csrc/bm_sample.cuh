@@ -116,5 +116,7 @@ inline size_t sample_smem_bytes(int bitmap_words) {
 cudaError_t launch_gather(const float* X, long long m, int n, const long long* idx, long long s, float* out,
                           Globals* g, cudaStream_t st);
 cudaError_t launch_sample(int np, const SampleArgs& a, int jobs, cudaStream_t st);
+// Kernels that a launch with these arguments consists of.
+inline int sample_kernels(const SampleArgs& a) { return a.wide ? 3 : 1; }
 
 }  // namespace bm

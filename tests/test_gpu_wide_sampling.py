@@ -68,3 +68,40 @@ def test_gather_checks_every_index(n):
         with pytest.raises(native.BigmeansError) as e:
             native.gather(X, idx)
         assert e.value.status == native.BM_EINVAL
+
+
+@pytest.mark.parametrize("rounds", [1, 3])
+def test_every_kernel_of_a_sampling_launch_is_counted(rounds):
+    """Three kernels per launch with many CTAs per job (here the first round's and the final sample;
+    the rounds drawn ahead take one), one with a CTA per job."""
+    X = torch.from_numpy(gaussian_mixture(60_000, 8, 5, seed=2)).cuda()
+    pol, bud = native.make_policy(s_min=500, s_max=9000, workers=3, passes=2), native.make_budget(rounds=rounds)
+    counts = []
+    try:
+        for impl in (0, 1):
+            native.set_sampler_impl(impl)
+            counts.append(native.fit(X, 5, pol, bud, seed=4)[2]["kernel_launches"])
+    finally:
+        native.set_sampler_impl(0)
+    assert counts[0] == counts[1] + 4
+
+
+def test_generations_start_again():
+    """A fit of more rounds than a table slot has generations clears both halves of its tables and goes
+    on: every sample is drawn by many CTAs (2 10^6 rows are too many for the bitmap), and the result
+    is that of one CTA per sample."""
+    rounds = 8300
+    X = torch.from_numpy(gaussian_mixture(40_000, 1, 4, seed=3)).cuda().repeat(50, 1).contiguous()
+    pol = native.make_policy(s_min=4100, s_max=4200, workers=1, passes=1)
+    bud = native.make_budget(rounds=rounds, max_lloyd=1)
+    outs = []
+    try:
+        for impl in (0, 1):
+            native.set_sampler_impl(impl)
+            outs.append(native.fit(X, 2, pol, bud, seed=8))
+    finally:
+        native.set_sampler_impl(0)
+    (C0, Y0, r0), (C1, Y1, r1) = outs
+    assert r0["rounds_done"] == rounds and r0["kernel_launches"] >= 4 * rounds
+    assert torch.equal(C0, C1) and torch.equal(Y0, Y1) and r0["f_full"] == r1["f_full"]
+    assert r0["accepts"] == r1["accepts"] and r0["L_sum"] == r1["L_sum"]
