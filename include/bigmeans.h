@@ -500,7 +500,8 @@ int32_t bm_get_big_clusters(void);
  * stream of bounded draws, in order of first occurrence).  impl 0 (default):
  * where the largest sample has at least 4096 rows and at most m / 2, many CTAs
  * per sample on open-addressing tables in device memory; else, and for the
- * samples a fit draws ahead while its workers run, one CTA per sample with a
+ * samples a fit draws ahead while its workers run and those of bm_sample with
+ * fewer than 8000 rows, one CTA per sample with a
  * shared-memory bitmap of the m indices where it fits (m up to about 1.37e6:
  * the bitmap and the per-chunk hash table within 200 KB); else one CTA per
  * sample on the tables; impl 1: always the last.

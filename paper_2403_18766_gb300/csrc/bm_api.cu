@@ -342,6 +342,10 @@ WorkerArgs make_args(const bm_fit_ctx* c, int mode, int parity = 0) {
 // Smallest largest sample drawn by many CTAs per job (below, one launch of a
 // CTA per job is as quick: fit of 10^4 x 2 with samples up to 2000).
 constexpr long long kWideMin = 4096;
+// The same where no rows are gathered (bm_sample) and the bitmap fits: 10^6
+// rows, us a call with one CTA and with many: s = 4096 82 and 92, 6000 85 and
+// 94, 8000 100 and 95, 20,000 137 and 96.
+constexpr long long kWideMinStep = 8000;
 int wide_chunks(const bm_fit_ctx* c) { return (int)((c->Tcap + kWideDraws - 1) / kWideDraws); }
 // Many CTAs per job: a table that half fills at most (2 s <= m keeps the
 // draws few), draw indices of 20 bits, jobs as a grid dimension.
@@ -384,7 +388,7 @@ bm_status make_sample_args(bm_fit_ctx* c, int mode, int jobs, int parity, bool a
     const long long words = (c->m + 31) / 32;
     const size_t sb = sample_smem_bytes((int)std::min<long long>(words, 1 << 30));
     const bool bitmap = !g_sample_tables.load() && words <= (1 << 30) && sb <= 200 * 1024;
-    a.wide = wide_sampling(c, jobs) && !(ahead && bitmap);
+    a.wide = wide_sampling(c, jobs) && !(bitmap && (ahead || (mode == kSampleStep && c->s_cap < kWideMinStep)));
     if (!a.wide && bitmap) a.bitmap_words = (int)words;
     if (a.bitmap_words > 0) return BM_OK;                 // no table
     if (a.wide) {
