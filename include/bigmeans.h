@@ -424,7 +424,7 @@ bm_status bm_assign_noalloc(const float* X_dev, int64_t m, int32_t n, const floa
  * f (the same FP32 direct-form definition, certified).
  *   impl 0 (default): by shape -- with n_pad = n rounded up to 4, 8, 16, 32 or
  *          64, the tensor-core pass when it applies and n_pad * k >= 256
- *          (n % 4 == 0) or 768 (other n) for m > 131,072, and when
+ *          (n % 4 == 0) or 768 (other n > 1) for m > 131,072, and when
  *          n % 4 == 0 and n_pad * k > 512 (n_pad <= 32) or 1600 for fewer
  *          rows; else the FP32-ALU pass;
  *   impl 1: always the FP32-ALU pass (register-tiled expanded form, certified,

@@ -414,12 +414,14 @@ int fullpass_impl_setting() { return g_fullpass_impl.load(); }
 // so the line lies at NP k = 256.  Widths that are no multiple of 4 come by
 // 1-D copies and are read word by word from shared memory, which moves it:
 //   10^6 x 63, k = 7: 109 / 124     1.5 10^6 x 21, k = 33: 115 / 95
+// One column is out: neighbouring centroids lie so close to each other that
+// most rows have several candidates (calls, us): 5 10^6 x 1, k = 200: 703 / 924
 // Up to 131,072 rows (about a tile per warpgroup) the start dominates and the
 // two are within 2 us of each other below NP k = 512 (NP <= 32) or 1600:
 //   5 10^4 x 16, k = 25: 15 / 15    5 10^4 x 16, k = 50: 19 / 15
 bool fullpass_prefers_tensor(long long m, int n, int np, int k) {
     const long long w = (long long)np * k;
-    if (n % 4 != 0) return m > 131072 && w >= 768;
+    if (n % 4 != 0) return n > 1 && m > 131072 && w >= 768;
     return m > 131072 ? w >= 256 : w > (np <= 32 ? 512 : 1600);
 }
 cudaError_t launch_fullpass(int np, const float* X, long long m, int n, const float* C, int k,
