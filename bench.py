@@ -413,7 +413,7 @@ def run_ours(args):
                  "frac": full_gbs / hbm_peak,
                  "traffic": traffic_full.get("dram_bytes_per_launch") if traffic_full else None,
                  "source_digest": digest_full,
-                 "kernel": ("tcx_fullpass_kernel<16> (tcgen05 split-TF32, certified, labels + f(C, X))"
+                 "kernel": ("tcx_fullpass_kernel<16> (tcgen05 split-BF16, certified, labels + f(C, X))"
                             if tensor_full else "fullpass_kernel<16> (FP32 ALU, certified, labels + f(C, X))"),
                  "algorithmic": f"m*n*4 = {bytes_full:.4g} bytes per launch (X read once)",
                  "avg_launch_us": t_full / max(n_full, 1) * 1e6, "peak_source": peak_src}

@@ -125,8 +125,10 @@ typedef struct {
                                assignment); Lloyd pts*k = assign_rows * k     */
     int64_t accepts;        /* |L|                                            */
     int64_t L_sum;          /* sum of L                                       */
-    int64_t rescored_rows;  /* rows whose FP32 expanded-form argmin was not
-                               certified and were re-scored in direct form    */
+    int64_t rescored_rows;  /* rows the certificate left more than one
+                               centroid for, decided in direct form: among
+                               all centroids (Lloyd, FP32-ALU pass) or among
+                               those left (tensor-core pass)                  */
     int64_t inexact_terms;  /* values truncated by the fixed-point grids      */
     double t_total_s;       /* wall time of the call                          */
     double t_worker_s;      /* device time of the worker-kernel launches

@@ -3,17 +3,18 @@
 // Algorithm 1 draws, for every worker and round, one sample to recompute
 // f_hat_w and one sample per pass (Sec. 4.1: "a new uniformly random sample
 // ... in each iteration").  None of them depends on clustering results, so
-// they are all drawn up front, one CTA per (worker, sample) job, and gathered
+// they are all drawn up front, a job per (worker, sample), and gathered
 // into contiguous padded rows that the worker kernel then reuses.
 //
 // A sample of size s is the first s distinct values among the bounded draws
-// r_0, r_1, ... of its Philox stream, in order of first occurrence.  When a
-// bitmap of the m values fits in shared memory, a job marks the values it has
+// r_0, r_1, ... of its Philox stream, in order of first occurrence.  Larger
+// samples are drawn by many CTAs each (sample_wide_*).  Else, when a bitmap of the m values fits in shared memory, a job marks the values it has
 // taken in that bitmap (sample_by_bitmap); otherwise it inserts its draws into
 // an open-addressing table in global memory whose slots hold
 // (generation << 32 | t): the generation of the job marks a slot as used, so
-// the table never needs clearing, and the value of a slot is draws[t].  A
-// draw t is kept when the slot of its value holds t itself (the least t).
+// the table is cleared only when its slots change between this form and that
+// of sample_wide_* (or the latter's generations run out), and the value of a
+// slot is draws[t].  A draw t is kept when the slot of its value holds t itself (the least t).
 #include <algorithm>
 #include <cstdint>
 

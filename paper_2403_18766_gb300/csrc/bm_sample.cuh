@@ -82,7 +82,7 @@ struct SampleArgs {
     unsigned int* draws; long long draws_stride;
     long long Tcap;
     unsigned long long* table; long long H; long long table_stride;
-    unsigned int gen_base;                     // generation of job 0 (tables are never cleared)
+    unsigned int gen_base;                     // generation of job 0 (a CTA per job)
     int bitmap_words;                          // > 0: draw with a shared-memory bitmap of the m
                                                // values ((m + 31) / 32 words) instead of the tables
     // many CTAs per job (sample_wide_*): per job `chunks` chunks of

@@ -137,7 +137,7 @@ __device__ __forceinline__ void tmem_dealloc(unsigned taddr, unsigned cols) {
 }
 
 // 32 lanes x 16 columns of 32-bit tensor-memory cells -> 16 registers per
-// thread (no wait; pair with wait_ld).
+// thread (no wait; pair with wait_ld16).
 __device__ __forceinline__ void ld16(unsigned taddr, unsigned (&r)[16]) {
     asm volatile(
         "tcgen05.ld.sync.aligned.32x32b.x16.b32 {%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, "
@@ -146,10 +146,9 @@ __device__ __forceinline__ void ld16(unsigned taddr, unsigned (&r)[16]) {
           "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
         : "r"(taddr));
 }
-__device__ __forceinline__ void wait_ld() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
 
 // ---------------------------------------------- epilogue helpers (g top-2)
-// Both tensor-core passes read, per row, g_j = fl(ccb_j - 2 acc_j) from the
+// The BF16 pass reads, per row, g_j = fl(ccb_j - 2 acc_j) from the
 // accumulator columns in chunks of 16 and keep the two least g (pass 1),
 // then a bit mask of the columns with g <= lim, i.e. below next_up(lim) (pass 2).
 

@@ -83,15 +83,8 @@ struct WorkerArgs {
 };
 
 struct Xch {
-    unsigned long long f_lo, f_hi;     // CTA partial of the exact objective
-    unsigned long long inexact, rescored;
-    long long wsum;                    // CTA sum of K-means++ weights
-    long long pot[4];                  // CTA partial candidate potentials
-    unsigned int maxbits;              // CTA max of D^2 bits
-    int cand[4];                       // candidate row found by this CTA, -1 if none
-    int stop;                          // rank-0 decision broadcast
-    int flag;                          // rank-0 flag broadcast
-    double fval;                       // rank-0 objective broadcast
+    int flag;                          // rank 0's deadline decision
+    int reserved[27];                  // (the limits of k and n count these bytes)
 };
 
 __host__ __device__ inline size_t align16(size_t v) { return (v + 15) & ~(size_t)15; }

@@ -1,18 +1,19 @@
 #pragma once
 // Fused Big-means worker kernel (template body; instantiated per padded
-// width NP in bm_worker_np*.cu): one thread-block cluster per competing
-// worker of Algorithm 1 (arXiv 2403.18766, Sec. 4.2-4.3).
+// width NP in bm_worker_np*.cu): one thread-block cluster, or a group of
+// clusters, per competing worker of Algorithm 1 (arXiv 2403.18766, Sec. 4.2-4.3).
 //
 // The samples of a round are drawn and gathered beforehand by the sampling
 // kernel.  A worker's sample is split into contiguous row slices, one per CTA
-// of its cluster.  Per pass the cluster re-seeds degenerate centroids with
-// greedy K-means++ (a3), runs Lloyd's iterations (a4-a6) and applies the
-// incumbent rule.  Cross-CTA exchange goes through distributed shared memory;
-// every cross-CTA dependency is separated by a hardware cluster barrier
-// (barrier.cluster, no spinning in this code).  All control flow that reaches
-// a cluster barrier is cluster-uniform: it only depends on kernel arguments
-// and on values every CTA reads after a barrier from the same place, so all
-// CTAs execute the same sequence of barriers.
+// of its clusters.  Per pass they re-seed degenerate centroids with greedy
+// K-means++ (a3), run Lloyd's iterations (a4-a6) and apply the incumbent rule.
+// Exchange within a cluster goes through distributed shared memory and hardware
+// cluster barriers (barrier.cluster); exchange within a group, and that of
+// K-means++, through global memory, in a group with a counter that a CTA polls
+// a bounded number of times (gsync).  All control flow that reaches a barrier
+// is uniform over the CTAs that meet there: it only depends on kernel arguments
+// and on values every CTA reads after a barrier from the same place, so all of
+// them execute the same sequence of barriers.
 #include <cstdint>
 #include <map>
 #include <mutex>
@@ -41,8 +42,7 @@ struct Sm {
     long long* red64;             // one per warp, + 1
     unsigned int* redu;           // one per warp
     CertC* cert;
-    long long* bcast;             // broadcast slots: 0 f, 1 stop, 2 M/pick, 3 base,
-                                  // 4 total, 5-7 candidates, 8 deadline flag
+    long long* bcast;             // values for the CTA: 2 K-means++ best, 3 its largest D^2, 8 deadline flag
     unsigned short* labs;         // rows_cta: label of each row of the CTA (first assignment)
     unsigned short* rowlist;      // rows_cta: the CTA's row offsets sorted by label
 };
@@ -294,7 +294,7 @@ struct Worker {
     // values when every value was split in two 64-bit halves and every row's
     // label compared.  A coordinate of at least 2^(gx + 71) (2^-24 of the
     // largest |x|) is a whole number of 2^(gx + 48) and needs one half; the
-    // others take the second half for their batch.  @BUCKET@
+    // others take the second half for their batch.
     __device__ bool bucket_sums(long long lo, long long hi, unsigned int& inex) {
         const int nrows = (int)(hi - lo);
         __syncthreads();                                   // labs and lcnt complete
@@ -573,7 +573,7 @@ struct Worker {
                             red_s32(owner_count(sold), -1);
                             lab_prev[srow] = snew;
                         }
-                                                for (int d = lane; d < n; d += 32) {
+                        for (int d = lane; d < n; d += 32) {
                             __int128 v;
                             ty.ok &= fixed_of(S[tile_at<NP>(srow, d)], g.gx, ty.inex, v);
                             add_words(owner_words(snew, d), v);
@@ -588,7 +588,7 @@ struct Worker {
     // idle: a short remainder (or a small sample's whole slice) is spread over
     // all warps instead of filling a few.
     template <int R>
-    __device__ __forceinline__ bool assign_trip(int want, long long t0, long long t1, int nwant, long long lo,
+    __device__ __forceinline__ void assign_trip(int want, long long t0, long long t1, int nwant, long long lo,
                                                 long long hi, int mode, const CertC& cc, const FastSum& fs,
                                                 Tally& ty) {
         if constexpr (R > 1)
@@ -597,7 +597,6 @@ struct Worker {
         const long long row0 = t0 + (long long)wid * 32 * R, nx0 = min(hi, t1 + (long long)wid * 32 * nwant);
         if (row0 < hi)
             assign_rows<R>(row0, lo, hi, nx0, min(hi, nx0 + 32 * nwant), mode, cc, fs, ty);
-        return true;
     }
     __device__ static int trip_rows(long long left) {        // R for the rows that are left
         constexpr int RT = RowsPerThread<NP>::v;
@@ -918,7 +917,7 @@ struct Worker {
     // leaves the row in candbuf.  One barrier per centroid is the only time
     // the CTAs wait for one another.
     static constexpr int kNoExp = 1 << 20;
-    static constexpr int kKppWords = 8 + 3 * kMaxWarps;     // of the 64 words of a CTA's slot
+    static_assert(8 + 3 * kMaxWarps <= 64, "a CTA's slot: totals, maxima and the sums of its warps");
     __device__ float* candbuf(int par, int l) const {       // in the (idle) sums: 24 NP bytes per cluster, k >= 2
         return reinterpret_cast<float*>(sm.OACC) + (par * 3 + l) * NP;
     }
@@ -1212,8 +1211,6 @@ struct Worker {
         __syncthreads();
     }
 };
-
-// trials > 3 would need more broadcast slots; the host caps it at 3.
 
 // BATCH: a launch for several fits, whose arguments are read from device
 // memory (p.batch[fit of the cluster]); otherwise the kernel parameter itself.
