@@ -36,14 +36,14 @@
 //
 // Threshold.  With the largest ||c||^2 in that bound, one far centroid would
 // make every row keep the centroids near it.  So the accumulator starts from
-// (1 - 2 gB) ||c_j||^2 (a hair less): then the squared distance D_j =
+// (1 - 2 gB) ||c_j||^2 (less by 0.005 gB, which covers its roundings): then the squared distance D_j =
 // ||x||^2 + ||c_j||^2 - 2 x.c_j is at least ||x||^2 + g_j - gB ||x||^2, and for
 // the centroid of the least g, g1, at most
-//   D <= ||x||^2 + g1 + gB (||x||^2 + 4.1 N),   N = ||c||^2 of that centroid.
+//   D <= ||x||^2 + g1 + gB (||x||^2 + 4.01 N),   N = ||c||^2 of that centroid.
 // N <= (||x|| + sqrt D)^2 <= 1.5 ||x||^2 + 3 D, hence (gB < 2^-12)
 //   D <= d1 = 1.006 (max(0, ||x||^2 + g1) + 7.2 gB ||x||^2),
 // and a centroid whose g exceeds g1 by more than
-//   thr = gB (2 ||x||^2 + 4.1 min(max ||c||^2, 1.5 ||x||^2 + 3 d1)) + gp2 d1
+//   thr = gB (2 ||x||^2 + 4.01 min(max ||c||^2, 1.5 ||x||^2 + 3 d1)) + gp2 d1
 // has a D larger by gp2 D and more, so a larger direct form (its relative
 // error is in gp2).  A gap below 2^-60 is never accepted (subnormal data), and
 // rows whose magnitudes come near the FP32 range keep all columns.  Up to 32
@@ -181,25 +181,6 @@ tcx_fullpass_kernel(const __grid_constant__ CUtensorMap tmap, const float* __res
     if (warp == kMma) tc::tmem_alloc(&tmem_slot, (unsigned)sh.tmem_cols);
     __syncthreads();
     const float* C = Cw + (long long)wsel * k * cw;
-    // copy of the CTA's it-th tile into stage s (the producer's lane 0)
-    auto copy_tile = [&](long long it, int s) {
-        const long long tile = blockIdx.x + it * gridDim.x;
-        if (sh.flat) {
-            const long long rows = min((long long)kTxRows, m - tile * kTxRows);
-            const unsigned bytes = (unsigned)(rows * n * 4) & ~15u;     // the rest by the row's thread
-            tc::expect_tx(&full[s], bytes);
-            if (bytes) tc::bulk_g2s(xs + (size_t)s * kStage, X + tile * kTxRows * n, bytes, &full[s]);
-        } else {
-            tc::expect_tx(&full[s], (unsigned)kStage);
-            for (int a = 0; a < K::atoms; ++a)
-                tc::tma_load_2d(xs + (size_t)s * kStage + (size_t)a * kTxAtomBytes, &tmap, 32 * a,
-                                (int)(tile * kTxRows), &full[s]);
-        }
-    };
-    long long issued = 0;             // producer: copies issued; MMA warp: tiles committed
-    if (warp == kProducer && lane == 0)                              // the first tiles are on their way meanwhile
-        for (; issued < S && blockIdx.x + issued * gridDim.x < (m + kTxRows - 1) / kTxRows; ++issued)
-            copy_tile(issued, (int)issued);
     // the FP32 copy of -c and the shift
     if (sh.cf)
         for (int e = tid; e < k * NP; e += kThreads) {
@@ -268,7 +249,7 @@ tcx_fullpass_kernel(const __grid_constant__ CUtensorMap tmap, const float* __res
                 if (shift) v = sub4(v, mu4[q]);
                 add(v.x); add(v.y); add(v.z); add(v.w);
             }
-        if (tid < sh.acc_stride) CC[tid] = tid < k ? cc * (1.f - 2.02f * gB) : __int_as_float(0x7f800000);
+        if (tid < sh.acc_stride) CC[tid] = tid < k ? cc * (1.f - 2.005f * gB) : __int_as_float(0x7f800000);
         const unsigned mx = __reduce_max_sync(0xffffffffu, __float_as_uint(up));
         if (lane == 0) redu[warp] = mx;
     }
@@ -298,16 +279,28 @@ tcx_fullpass_kernel(const __grid_constant__ CUtensorMap tmap, const float* __res
 
     unsigned __int128 facc = 0;
     unsigned int inex = 0, resc = 0;
+    long long issued = 0;             // producer: copies issued; MMA warp: tiles committed
     if (warp == kProducer) {
         // ---------------------------------------------------------- producer
         if (lane == 0) {
-            long long it = issued;
-            int s = (int)(it % S);
-            unsigned ph = (unsigned)(it / S) & 1u;          // (it / S) & 1, kept incrementally
+            long long it = 0;
+            int s = 0;
+            unsigned ph = 0;                                // (it / S) & 1, kept incrementally
             for (;; ++it) {
-                if (blockIdx.x + it * grid >= ntiles) break;
+                const long long tile = blockIdx.x + it * grid;
+                if (tile >= ntiles) break;
                 if (it >= S && !tc::wait(&empty[s], ph ^ 1u, abort, g, sh.wait)) break;
-                copy_tile(it, s);
+                if (sh.flat) {
+                    const long long rows = min((long long)kTxRows, m - tile * kTxRows);
+                    const unsigned bytes = (unsigned)(rows * n * 4) & ~15u;     // the rest by the row's thread
+                    tc::expect_tx(&full[s], bytes);
+                    if (bytes) tc::bulk_g2s(xs + (size_t)s * kStage, X + tile * kTxRows * n, bytes, &full[s]);
+                } else {
+                    tc::expect_tx(&full[s], (unsigned)kStage);
+                    for (int a = 0; a < K::atoms; ++a)
+                        tc::tma_load_2d(xs + (size_t)s * kStage + (size_t)a * kTxAtomBytes, &tmap, 32 * a,
+                                        (int)(tile * kTxRows), &full[s]);
+                }
                 if (++s == S) { s = 0; ph ^= 1u; }
             }
             issued = it;
@@ -347,9 +340,9 @@ tcx_fullpass_kernel(const __grid_constant__ CUtensorMap tmap, const float* __res
         auto epilogue = [&](auto shifted) __attribute__((always_inline)) {
         const Grids gr = grids_from_maxbits(g->maxbits);
         const float cmax2 = __uint_as_float(__reduce_max_sync(0xffffffffu, lane < kThreads / 32 ? redu[lane] : 0u));
-        // (each constant of the threshold has 2^-9 of itself to spare for roundings)
-        const float k_max = fmaxf(4.11f * gB * cmax2, 0x1p-60f);
-        const float k_gp = gp2 * (1.f + 0x1p-9f), k_own = 12.4f * gB + k_gp;
+        // (each constant of the threshold has 2^-10 of itself to spare for roundings)
+        const float k_max = fmaxf(4.02f * gB * cmax2, 0x1p-60f);
+        const float k_gp = gp2 * (1.f + 0x1p-10f), k_own = 12.4f * gB + k_gp;
         const int b = warp >> 2, q4 = warp & 3;
         const int r = q4 * 32 + lane;                        // row within the tile = TMEM lane
         unsigned char* xrow = xb + (size_t)b * kStage + r * 128;
@@ -429,7 +422,7 @@ tcx_fullpass_kernel(const __grid_constant__ CUtensorMap tmap, const float* __res
             if constexpr (decltype(shifted)::value) xn2 = __fmul_ru(xn2, 1.f + 0x1p-21f);
             // what the threshold takes from ||x||^2
             const float d_lo = __fmul_ru(7.3f * gB, xn2);
-            const float t_max = __fmaf_ru(2.01f * gB, xn2, k_max);
+            const float t_max = __fmaf_ru(2.002f * gB, xn2, k_max);
             const bool sane = t_max < 0x1p106f;               // ||x||^2 + 2 cmax^2 below 2^122; else: every column
             const float t_own = fmaxf(__fmul_ru(8.2f * gB, xn2), 0x1p-60f);
             // 2. the accumulator: least g, then the columns within the threshold
