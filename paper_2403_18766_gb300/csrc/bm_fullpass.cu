@@ -408,12 +408,12 @@ int fullpass_impl_setting() { return g_fullpass_impl.load(); }
 // barriers) and little per column, and it starts slower.  Measured on GB300,
 // ALU against tensor cores, us (kernel, rows not in L2):
 //   10^6 x 2,  k = 5:  21 / 33      10^6 x 8,  k = 10: 27 / 33
-//   10^6 x 16, k = 25: 44 / 36      10^6 x 8,  k = 100: 81 / 46
-//   4 10^6 x 32, k = 10: 177 / 136  4 10^6 x 32, k = 50: 421 / 173
-//   10^6 x 64, k = 10: 111 / 70     10^7 x 64, k = 100: 4137 / 857
+//   10^6 x 16, k = 25: 44 / 33      10^6 x 8,  k = 100: 81 / 46
+//   4 10^6 x 32, k = 10: 177 / 136  4 10^6 x 32, k = 50: 421 / 181
+//   10^6 x 64, k = 10: 111 / 70     10^7 x 64, k = 100: 4137 / 879
 // so the line lies at NP k = 256.  Widths that are no multiple of 4 come by
 // 1-D copies and are read word by word from shared memory, which moves it:
-//   10^6 x 63, k = 7: 109 / 124     1.5 10^6 x 21, k = 33: 115 / 95
+//   10^6 x 63, k = 7: 109 / 124     1.5 10^6 x 21, k = 33: 115 / 97
 // One column is out: neighbouring centroids lie so close to each other that
 // most rows have several candidates (calls, us): 5 10^6 x 1, k = 200: 703 / 924
 // Up to 131,072 rows (about a tile per warpgroup) the start dominates and the

@@ -63,8 +63,8 @@
 // every column costs less than the FP32-ALU pass, and nothing is shifted.
 // Measured, kernel alone, rows with a mean of 300 standard deviations: 10^6 x
 // 16, k = 200 2,110 -> 93 us; 2 10^6 x 32, k = 50 758 -> 99 us; 2 10^6 x 64, k =
-// 100 2,650 -> 207 us; centred rows, which pay for the test, 91 -> 93, 95 -> 97
-// and 189 -> 193 us.
+// 100 2,650 -> 207 us.  With both, centred rows take 1% longer (10^7 x 64, k =
+// 100: 867 -> 879 us).
 //
 // CTA roles (one CTA per SM, persistent over tiles blockIdx.x + i grid): the
 // warp after the epilogue warps issues the copies of X, the next one the
@@ -80,12 +80,12 @@
 // of n floats (odd n: no bank conflicts).
 //
 // What bounds it: latency within a tile (wait, split, MMA, tensor-memory load,
-// distance are one chain per group; 38% issue, 21% of the DRAM cycles at 10^6
-// x 16, k = 25), hence as many groups as fit.  The former passes (three
+// distance are one chain per group; 48% issue, 25% of the DRAM rate at 10^6 x
+// 16, k = 25), hence as many groups as fit.  The former passes (three
 // split-TF32 products, two reads of the accumulator with a compare and a
 // select per column, rows rebuilt from two tiles) issued 2-3 times as many
-// instructions: 10^7 x 64, k = 100: 2.83 ms then, 0.86 ms now (2.99 TB/s of
-// rows); 4 10^6 x 32, k = 50: 228 and 173 us; 10^6 x 16, k = 25: 49 and 36 us.
+// instructions: 10^7 x 64, k = 100: 2.83 ms then, 0.88 ms now (2.9 TB/s of
+// rows); 4 10^6 x 32, k = 50: 228 and 181 us; 10^6 x 16, k = 25: 49 and 33 us.
 #include <algorithm>
 #include <atomic>
 #include <cstdint>
